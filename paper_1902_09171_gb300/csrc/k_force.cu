@@ -292,8 +292,7 @@ __global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), density_min_ctas(TPA))
     const int c = a.tile_cell[t];
     if (a.status[c] != 0 || !a.active[c]) return;
     __shared__ ShiftTab s_tab;
-    __shared__ float s_H[8];
-    rc_load_shifts(s_tab, s_H, a.Hf, c);
+    rc_load_shifts(s_tab, a.shift, c);
 
     const int at = threadIdx.x / lanes_of(TPA), sub = threadIdx.x % lanes_of(TPA);
     const int n = a.cell_n[c], off = a.cell_off[c];
@@ -374,8 +373,7 @@ __global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), force_min_ctas(TPA)) k
     const int c = a.tile_cell[t];
     if (a.status[c] != 0 || !a.active[c]) return;
     __shared__ ShiftTab s_tab;
-    __shared__ float s_H[8];
-    rc_load_shifts(s_tab, s_H, a.Hf, c);
+    rc_load_shifts(s_tab, a.shift, c);
 
     const int at = threadIdx.x / lanes_of(TPA), sub = threadIdx.x % lanes_of(TPA);
     const int n = a.cell_n[c], off = a.cell_off[c];
@@ -615,8 +613,7 @@ __global__ void __launch_bounds__(RC_TILE) k_static_pk1(KParams p, KArrays a, in
     const int c = a.tile_cell[t];
     if (a.status[c] != 0 || !a.active[c]) return;
     __shared__ ShiftTab s_tab;
-    __shared__ float s_H[8];
-    rc_load_shifts(s_tab, s_H, a.Hf, c);
+    rc_load_shifts(s_tab, a.shift, c);
     const float *m = mcell + 6 * c;
     const float m00 = m[0], m01 = m[1], m02 = m[2], m11 = m[3], m12 = m[4], m22 = m[5];
     const int n = a.cell_n[c], off = a.cell_off[c];
@@ -702,11 +699,11 @@ template <int POT, bool M6, bool STG, bool SAMPLE>
 void launch_force_tpa(const KParams &p, const KArrays &a, int cur, int n_tiles, int tpa, int mode, int slot,
                       int step_index, int smem, cudaStream_t s) {
     switch (tpa) {
-    case 0: rc_launch_pdl(k_force<POT, 0, M6, STG, SAMPLE>, pair_grid(p), RC_TILE * 1, smem, s, p, a, cur, mode, slot, step_index); break;
-    case 1: rc_launch_pdl(k_force<POT, 1, M6, STG, SAMPLE>, pair_grid(p), RC_TILE * 1, smem, s, p, a, cur, mode, slot, step_index); break;
-    case 2: rc_launch_pdl(k_force<POT, 2, M6, STG, SAMPLE>, pair_grid(p), RC_TILE * 2, smem, s, p, a, cur, mode, slot, step_index); break;
-    case 4: rc_launch_pdl(k_force<POT, 4, M6, STG, SAMPLE>, pair_grid(p), RC_TILE * 4, smem, s, p, a, cur, mode, slot, step_index); break;
-    default: rc_launch_pdl(k_force<POT, 8, M6, STG, SAMPLE>, pair_grid(p), RC_TILE * 8, smem, s, p, a, cur, mode, slot, step_index); break;
+    case 0: rc_launch_pdl(k_force<POT, 0, M6, STG, SAMPLE>, pair_grid(p), RC_TILE * 1, smem, s, 1, p, a, cur, mode, slot, step_index); break;
+    case 1: rc_launch_pdl(k_force<POT, 1, M6, STG, SAMPLE>, pair_grid(p), RC_TILE * 1, smem, s, 1, p, a, cur, mode, slot, step_index); break;
+    case 2: rc_launch_pdl(k_force<POT, 2, M6, STG, SAMPLE>, pair_grid(p), RC_TILE * 2, smem, s, 1, p, a, cur, mode, slot, step_index); break;
+    case 4: rc_launch_pdl(k_force<POT, 4, M6, STG, SAMPLE>, pair_grid(p), RC_TILE * 4, smem, s, 1, p, a, cur, mode, slot, step_index); break;
+    default: rc_launch_pdl(k_force<POT, 8, M6, STG, SAMPLE>, pair_grid(p), RC_TILE * 8, smem, s, 1, p, a, cur, mode, slot, step_index); break;
     }
 }
 
@@ -722,11 +719,11 @@ void launch_force_pot(const KParams &p, const KArrays &a, int cur, int n_tiles, 
 template <bool M6, bool STG>
 void launch_density_m(const KParams &p, const KArrays &a, int cur, int n_tiles, int tpa, int smem, cudaStream_t s) {
     switch (tpa) {
-    case 0: rc_launch_pdl(k_density<0, M6, STG>, pair_grid(p), RC_TILE * 1, smem, s, p, a, cur); break;
-    case 1: rc_launch_pdl(k_density<1, M6, STG>, pair_grid(p), RC_TILE * 1, smem, s, p, a, cur); break;
-    case 2: rc_launch_pdl(k_density<2, M6, STG>, pair_grid(p), RC_TILE * 2, smem, s, p, a, cur); break;
-    case 4: rc_launch_pdl(k_density<4, M6, STG>, pair_grid(p), RC_TILE * 4, smem, s, p, a, cur); break;
-    default: rc_launch_pdl(k_density<8, M6, STG>, pair_grid(p), RC_TILE * 8, smem, s, p, a, cur); break;
+    case 0: rc_launch_pdl(k_density<0, M6, STG>, pair_grid(p), RC_TILE * 1, smem, s, 1, p, a, cur); break;
+    case 1: rc_launch_pdl(k_density<1, M6, STG>, pair_grid(p), RC_TILE * 1, smem, s, 1, p, a, cur); break;
+    case 2: rc_launch_pdl(k_density<2, M6, STG>, pair_grid(p), RC_TILE * 2, smem, s, 1, p, a, cur); break;
+    case 4: rc_launch_pdl(k_density<4, M6, STG>, pair_grid(p), RC_TILE * 4, smem, s, 1, p, a, cur); break;
+    default: rc_launch_pdl(k_density<8, M6, STG>, pair_grid(p), RC_TILE * 8, smem, s, 1, p, a, cur); break;
     }
 }
 

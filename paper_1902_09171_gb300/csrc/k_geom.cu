@@ -11,21 +11,18 @@ __device__ __forceinline__ double det3(const double *A) {
     return A[0] * (A[4] * A[8] - A[5] * A[7]) - A[1] * (A[3] * A[8] - A[5] * A[6]) + A[2] * (A[3] * A[7] - A[4] * A[6]);
 }
 
-// one thread per cell
-__global__ void k_deform(const double *__restrict__ Fin, double *H, double *Rprev, double *Qo, double *Ro,
-                         double *Fst, double *dR, const double *__restrict__ H0, float *Hf, float *Hif, int *status,
-                         int *need_rebuild, int *nbins, const int *bin_cap, const int *active, double rlist,
-                         int n_cells) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n_cells) return;
+// cell c by one thread; false when the cell keeps its state
+__device__ bool deform_cell(int c, const double *__restrict__ Fin, double *H, double *Rprev, double *Qo, double *Ro,
+                            double *Fst, double *dR, const double *__restrict__ H0, float *Hf, float *Hif, int *status,
+                            int *need_rebuild, int *nbins, const int *bin_cap, const int *active, double rlist) {
     double *dRc = dR + 9 * c;
     for (int k = 0; k < 9; k++) dRc[k] = (k % 4 == 0) ? 1.0 : 0.0;  // identity unless the cell is updated
-    if (status[c] != 0 || !active[c]) return;  // inactive cells keep box, R(t-1) and atoms
+    if (status[c] != 0 || !active[c]) return false;  // inactive cells keep box, R(t-1) and atoms
     double F[9];
     for (int k = 0; k < 9; k++) F[k] = Fin[9 * c + k];
     if (!(det3(F) > 0.0)) {
         atomicCAS(&status[c], 0, RC_EDEGEN);
-        return;
+        return false;
     }
     // modified Gram-Schmidt on the columns a_0, a_1, a_2 of F (Sec. 2.1); the
     // norms make the diagonal of R positive.
@@ -42,7 +39,7 @@ __global__ void k_deform(const double *__restrict__ Fin, double *H, double *Rpre
         const double nrm = sqrt(v0 * v0 + v1 * v1 + v2 * v2);
         if (!(nrm > 0.0)) {
             atomicCAS(&status[c], 0, RC_EDEGEN);
-            return;
+            return false;
         }
         R[3 * j + j] = nrm;
         q[j][0] = v0 / nrm;
@@ -71,7 +68,7 @@ __global__ void k_deform(const double *__restrict__ Fin, double *H, double *Rpre
     for (int k = 0; k < 3; k++)
         if (!(w[k] >= 2.0 * rlist)) {
             atomicCAS(&status[c], 0, RC_EBOX);
-            return;
+            return false;
         }
     int nb[3];
     for (int k = 0; k < 3; k++) nb[k] = (int)floor(2.0 * w[k] / rlist);  // bins at least r_list / 2 wide
@@ -111,6 +108,27 @@ __global__ void k_deform(const double *__restrict__ Fin, double *H, double *Rpre
     nbins[4 * c + 1] = nb[1];
     nbins[4 * c + 2] = nb[2];
     need_rebuild[c] = 1;
+    return true;
+}
+
+// one warp per cell: lane 0 the deformation, then lane k entry k of the new box's shift table
+constexpr int DEFORM_WARPS = 4;
+__global__ void __launch_bounds__(32 * DEFORM_WARPS)
+    k_deform(const double *__restrict__ Fin, double *H, double *Rprev, double *Qo, double *Ro, double *Fst, double *dR,
+             const double *__restrict__ H0, float *Hf, float *Hif, float4 *shift, int *status, int *need_rebuild,
+             int *nbins, const int *bin_cap, const int *active, double rlist, int n_cells) {
+    const int c = blockIdx.x * DEFORM_WARPS + threadIdx.x / 32, lane = threadIdx.x & 31;
+    if (c >= n_cells) return;
+    int done = 0;
+    if (lane == 0)
+        done = deform_cell(c, Fin, H, Rprev, Qo, Ro, Fst, dR, H0, Hf, Hif, status, need_rebuild, nbins, bin_cap, active,
+                           rlist);
+    __syncwarp();
+    if (__shfl_sync(0xffffffffu, done, 0) && lane < RC_SLOTS) rc_build_shift(shift + (size_t)c * RC_SHIFT_W, Hf + 8 * c, lane);
+}
+
+__global__ void k_shift(const float *Hf, float4 *shift, int c) {
+    if (threadIdx.x < RC_SLOTS) rc_build_shift(shift + (size_t)c * RC_SHIFT_W, Hf + 8 * c, threadIdx.x);
 }
 
 // x <- Delta R x (FP64 arithmetic on the FP32 positions); one thread per atom slot
@@ -265,11 +283,14 @@ __global__ void k_advance(unsigned long long *evals, const int *active, int n_ce
 }  // namespace
 
 void rc_launch_deform_impl(const double *F, double *H, double *Rprev, double *Q, double *R, double *Fst, double *dR,
-                           const double *H0, float *Hf, float *Hif, int *status, int *need_rebuild, int *nbins,
-                           const int *bin_cap, const int *active, double rlist, int n_cells, cudaStream_t s) {
-    k_deform<<<(n_cells + 127) / 128, 128, 0, s>>>(F, H, Rprev, Q, R, Fst, dR, H0, Hf, Hif, status, need_rebuild,
-                                                   nbins, bin_cap, active, rlist, n_cells);
+                           const double *H0, float *Hf, float *Hif, float4 *shift, int *status, int *need_rebuild,
+                           int *nbins, const int *bin_cap, const int *active, double rlist, int n_cells,
+                           cudaStream_t s) {
+    k_deform<<<(n_cells + DEFORM_WARPS - 1) / DEFORM_WARPS, 32 * DEFORM_WARPS, 0, s>>>(
+        F, H, Rprev, Q, R, Fst, dR, H0, Hf, Hif, shift, status, need_rebuild, nbins, bin_cap, active, rlist, n_cells);
 }
+
+void rc_launch_shift(const float *Hf, float4 *shift, int c, cudaStream_t s) { k_shift<<<1, 32, 0, s>>>(Hf, shift, c); }
 
 void rc_launch_remap(const KArrays &a, const double *dR, int cur, int n_tiles, cudaStream_t s) {
     k_remap<<<n_tiles, RC_TILE, 0, s>>>(a, dR, cur);

@@ -14,8 +14,9 @@
 //     candidates of an atom lie in the 5 x 5 x 5 bins around its own.
 //   * Verlet list: per tile, [max_nb/4][TILE] groups of four int32 entries
 //     j_global | (image << 27) (one 16-byte load per lane per group, coalesced
-//     across the tile); the image code 0..26 selects one of the 27 periodic
-//     shift vectors of the cell.
+//     across the tile); the image slot 0..26 selects one of the 27 periodic
+//     shift vectors of the cell.  The last group is filled up with null entries
+//     (slot 27), whose displacement is far beyond any cutoff.
 //   * Per-cell FP64 state: box H, stretch R(t-1), Q, R, F of the last
 //     deformation, Philox force-evaluation counter, status word.
 #pragma once
@@ -59,6 +60,7 @@ struct KArrays {
     const int *cell_n, *cell_off, *tile_cell, *cell_tile0;
     const float *Hf;     // 8 floats per cell: h00 h01 h02 h11 h12 h22 . .
     const float *Hif;    // inverse, same layout
+    const float4 *shift; // periodic shift tables, RC_SHIFT_W entries per cell
     const int *nbins;    // 4 ints per cell
     const int *bin_off;  // first bin slot per cell
     int *bin_start;      // bin_off[c] .. + nbins+1
@@ -75,7 +77,8 @@ struct KArrays {
     float4 *v, *xref, *xr, *f;
     int *tag;
     int4 *partner;       // cell-local indices, -1 = none
-    int *nbr, *nnb, *bin_of;
+    int *nbr, *nnb;
+    int *bin_of;         // packed bin: b0 << 20 | b1 << 10 | b2 (each below 1024: at least 4 bins per axis)
     // sort scratch
     float4 *x_tmp, *v_tmp;
     int *tag_tmp, *newpos, *oldidx, *binid;
@@ -133,31 +136,44 @@ __device__ __forceinline__ void rc_set_status(int *status, int cell, int code) {
 // Images are numbered by slot k = (code + 14) mod 27 of the image code
 // code = (sx+1) + 3(sy+1) + 9(sz+1): the central image (code 13) is slot 0, so
 // a list entry j | k << RC_IDX_BITS of the central image is the bare index j.
+// Slot 27 is the null entry that fills up a list's last group: its shift puts
+// the neighbour 1e18 length units away.
+//
+// The tables belong to the box: k_deform writes them (FP64, which this GPU runs
+// at 1/64 of the FP32 rate) and the pair kernels copy theirs to shared memory.
+// Built by every CTA of every launch instead, they kept each CTA's first
+// barrier waiting for 27 threads of FP64 work (SHIFT_FIGURES).
+constexpr int RC_SLOT_CENTRAL = 0;
+constexpr unsigned RC_SLOT_NULL = 27;
+constexpr int RC_SLOTS = 28, RC_SHIFT_W = 2 * RC_SLOTS;
 struct ShiftTab {
-    float4 a[27], b[27];
+    float4 a[RC_SLOTS], b[RC_SLOTS];
 };
 
-constexpr int RC_SLOT_CENTRAL = 0;
 __host__ __device__ __forceinline__ int rc_image_slot(int sx, int sy, int sz) {
     return ((sx + 1) + 3 * (sy + 1) + 9 * (sz + 1) + 14) % 27;
 }
 
-__device__ __forceinline__ void rc_build_shift(ShiftTab &T, const float *H, int slot) {
+// entry `slot` of the table of the box H (upper triangular, h00 h01 h02 h11 h12 h22)
+__device__ __forceinline__ void rc_build_shift(float4 *tab, const float *H, int slot) {
+    if (slot == (int)RC_SLOT_NULL) {
+        tab[slot] = make_float4(1e18f, 1e18f, 1e18f, 0.f);
+        tab[RC_SLOTS + slot] = make_float4(0.f, 0.f, 0.f, 0.f);
+        return;
+    }
     const int code = (slot + 13) % 27;
     const double sx = (double)(code % 3 - 1), sy = (double)((code / 3) % 3 - 1), sz = (double)(code / 9 - 1);
     const double hx = (double)H[0] * sx + (double)H[1] * sy + (double)H[2] * sz;
     const double hy = (double)H[3] * sy + (double)H[4] * sz;
     const double hz = (double)H[5] * sz;
     const float fx = (float)hx, fy = (float)hy, fz = (float)hz;
-    T.a[slot] = make_float4(fminf(fx, 0.f), fminf(fy, 0.f), fminf(fz, 0.f), (float)(hx - fx));
-    T.b[slot] = make_float4(fmaxf(fx, 0.f), fmaxf(fy, 0.f), fmaxf(fz, 0.f), (float)(hy - fy));
+    tab[slot] = make_float4(fminf(fx, 0.f), fminf(fy, 0.f), fminf(fz, 0.f), (float)(hx - fx));
+    tab[RC_SLOTS + slot] = make_float4(fmaxf(fx, 0.f), fmaxf(fy, 0.f), fmaxf(fz, 0.f), (float)(hy - fy));
 }
 
-// fill the table from cell c's box (call with all threads; syncs)
-__device__ __forceinline__ void rc_load_shifts(ShiftTab &T, float *s_H, const float *Hf, int c) {
-    if (threadIdx.x < 6) s_H[threadIdx.x] = Hf[8 * c + threadIdx.x];
-    __syncthreads();
-    if (threadIdx.x < 27) rc_build_shift(T, s_H, threadIdx.x);
+// cell c's table to shared memory (call with all threads; syncs)
+__device__ __forceinline__ void rc_load_shifts(ShiftTab &T, const float4 *shift, int c) {
+    if (threadIdx.x < RC_SHIFT_W) T.a[threadIdx.x] = shift[(size_t)c * RC_SHIFT_W + threadIdx.x];
     __syncthreads();
 }
 
@@ -190,19 +206,24 @@ __device__ __forceinline__ float3 rc_disp_central(const float4 &xi, const float4
 __device__ __forceinline__ void rc_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void rc_pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// cluster > 1: the grid (a multiple of it) runs in thread-block clusters of that many CTAs.
 template <class... KArgs, class... Args>
-void rc_launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+void rc_launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, int cluster,
                    Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = cluster;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
@@ -217,7 +238,7 @@ struct FireState {
 
 // host-side launchers (defined in the kernel translation units)
 void rc_launch_sort(const KParams &p, const KArrays &a, int cur, int n_cells, cudaStream_t s);
-void rc_launch_nlist(const KParams &p, const KArrays &a, int cur, int n_tiles, cudaStream_t s);
+void rc_launch_nlist(const KParams &p, const KArrays &a, int cur, int n_cells, cudaStream_t s);
 // stage_atoms > 0: every CTA first copies its whole r-cell (stage_atoms = the
 // largest cell of the batch) into shared memory and gathers neighbours there
 void rc_launch_density(const KParams &p, const KArrays &a, int cur, int n_tiles, int tpa, int stage_atoms,
@@ -227,8 +248,10 @@ void rc_launch_force(const KParams &p, const KArrays &a, int cur, int n_tiles, i
 int rc_stage_max_atoms();
 void rc_prepare_staged(int max_cell_atoms);
 void rc_launch_deform_impl(const double *F, double *H, double *Rprev, double *Q, double *R, double *Fst, double *dR,
-                           const double *H0, float *Hf, float *Hif, int *status, int *need_rebuild, int *nbins,
-                           const int *bin_cap, const int *active, double rlist, int n_cells, cudaStream_t s);
+                           const double *H0, float *Hf, float *Hif, float4 *shift, int *status, int *need_rebuild,
+                           int *nbins, const int *bin_cap, const int *active, double rlist, int n_cells, cudaStream_t s);
+// the shift table of cell c from its box
+void rc_launch_shift(const float *Hf, float4 *shift, int c, cudaStream_t s);
 void rc_launch_remap(const KArrays &a, const double *dR, int cur, int n_tiles, cudaStream_t s);
 void rc_launch_stress(const double *series, int n_avg, int series_cap, const double *H, const double *Q,
                       const double *F, double pconv, double *rot_scratch, double *sig_fem, double *sig_se,

@@ -39,6 +39,7 @@ struct rcell_ctx {
     double *d_H = nullptr, *d_H0 = nullptr, *d_Rprev = nullptr, *d_Q = nullptr, *d_R = nullptr, *d_F = nullptr;
     double *d_dR = nullptr, *d_Fin = nullptr;
     float *d_Hf = nullptr, *d_Hif = nullptr;
+    float4 *d_shift = nullptr;  // periodic shift tables (RC_SHIFT_W per cell)
     int *d_nbins = nullptr, *d_bin_cap = nullptr;
     unsigned long long *d_evals = nullptr;
     double *d_sig_fem = nullptr, *d_sig_se = nullptr, *d_sig_md = nullptr, *d_P = nullptr;
@@ -144,7 +145,7 @@ int stage_atoms(const rcell_ctx *c) {
 long enqueue_step(rcell_ctx *c, int mode, int slot, int step_index) {
     long k = 0;
     rc_launch_sort(c->kp, c->ka, c->cur, c->n_cells, c->stream);
-    rc_launch_nlist(c->kp, c->ka, c->cur, c->n_tiles, c->stream);
+    rc_launch_nlist(c->kp, c->ka, c->cur, c->n_cells, c->stream);
     k += 2;
     if (c->kp.pot == RC_POT_SC) {
         rc_launch_density(c->kp, c->ka, c->cur, c->n_tiles, c->tpa, stage_atoms(c), c->stream);
@@ -337,6 +338,7 @@ int rcell_create(const rcell_params *params, int n_cells, const rcell_init *cell
     CKC(c, dalloc(L, &c->d_Fin, 9 * (size_t)n_cells));
     CKC(c, dalloc(L, &c->d_Hf, 8 * (size_t)n_cells));
     CKC(c, dalloc(L, &c->d_Hif, 8 * (size_t)n_cells));
+    CKC(c, dalloc(L, &c->d_shift, RC_SHIFT_W * (size_t)n_cells));
     CKC(c, dalloc(L, &c->d_sig_fem, 6 * (size_t)n_cells));
     CKC(c, dalloc(L, &c->d_sig_se, 6 * (size_t)n_cells));
     CKC(c, dalloc(L, &c->d_sig_md, 6 * (size_t)n_cells));
@@ -365,6 +367,7 @@ int rcell_create(const rcell_params *params, int n_cells, const rcell_init *cell
     A.cell_tile0 = d_cell_tile0;
     A.Hf = c->d_Hf;
     A.Hif = c->d_Hif;
+    A.shift = c->d_shift;
     A.nbins = c->d_nbins;
     A.bin_off = d_bin_off;
     A.evals = c->d_evals;
@@ -415,7 +418,7 @@ int rcell_create(const rcell_params *params, int n_cells, const rcell_init *cell
     CKC(c, cudaMemcpy(c->d_Rprev, hI.data(), sizeof(double) * 9 * n_cells, cudaMemcpyHostToDevice));
     CKC(c, cudaMemcpy(c->d_Fin, hI.data(), sizeof(double) * 9 * n_cells, cudaMemcpyHostToDevice));
     // initial box: the deformation kernel with F = I sets H = H0, the FP32 box copies and the bins
-    rc_launch_deform_impl(c->d_Fin, c->d_H, c->d_Rprev, c->d_Q, c->d_R, c->d_F, c->d_dR, c->d_H0, c->d_Hf, c->d_Hif,
+    rc_launch_deform_impl(c->d_Fin, c->d_H, c->d_Rprev, c->d_Q, c->d_R, c->d_F, c->d_dR, c->d_H0, c->d_Hf, c->d_Hif, c->d_shift,
                           A.status, A.need_rebuild, c->d_nbins, c->d_bin_cap, A.active, c->rlist, n_cells, c->stream);
     CKC(c, cudaGetLastError());
     int st = first_status(c);
@@ -439,7 +442,7 @@ int rcell_set_deformation(rcell_ctx *c, const double *F, int where) {
     } else if (where != RC_DEVICE) {
         return fail(c, RC_EINVAL, "where");
     }
-    rc_launch_deform_impl(dF, c->d_H, c->d_Rprev, c->d_Q, c->d_R, c->d_F, c->d_dR, c->d_H0, c->d_Hf, c->d_Hif,
+    rc_launch_deform_impl(dF, c->d_H, c->d_Rprev, c->d_Q, c->d_R, c->d_F, c->d_dR, c->d_H0, c->d_Hf, c->d_Hif, c->d_shift,
                           c->ka.status, c->ka.need_rebuild, c->d_nbins, c->d_bin_cap, c->ka.active, c->rlist, c->n_cells, c->stream);
     rc_launch_remap(c->ka, c->d_dR, c->cur, c->n_tiles, c->stream);
     CKC(c, cudaGetLastError());
@@ -753,7 +756,7 @@ int rcell_stress_static(rcell_ctx *c, double *sigma, double *P, int where) {
     }
     rc_launch_static_prep(c->d_H, c->d_H0, c->d_mcell, c->d_pk_acc, nc, c->stream);
     rc_launch_sort(c->kp, c->ka, c->cur, nc, c->stream);
-    rc_launch_nlist(c->kp, c->ka, c->cur, c->n_tiles, c->stream);
+    rc_launch_nlist(c->kp, c->ka, c->cur, c->n_cells, c->stream);
     if (c->kp.pot == RC_POT_SC) rc_launch_density(c->kp, c->ka, c->cur, c->n_tiles, 1, 0, c->stream);
     rc_launch_static_pk1(c->kp, c->ka, c->cur, c->n_tiles, c->d_mcell, c->d_pk_acc, c->stream);
     rc_launch_static_finish(c->d_pk_acc, c->d_H0, c->d_Q, c->d_F, pconv_of(c->prm.units), c->d_P, c->d_sig_fem,
@@ -848,6 +851,8 @@ int rcell_restore(rcell_ctx *c, int cell, const void *buf, size_t bytes) {
     CKC(c, cudaMemcpy(c->d_Hif + 8 * cell, p, sizeof(float) * 8, cudaMemcpyHostToDevice)); p += sizeof(float) * 8;
     CKC(c, cudaMemcpy(c->d_nbins + 4 * cell, p, sizeof(int) * 4, cudaMemcpyHostToDevice)); p += sizeof(int) * 4;
     CKC(c, cudaMemcpy(c->d_evals + cell, p, sizeof(unsigned long long), cudaMemcpyHostToDevice));
+    rc_launch_shift(c->d_Hf, c->d_shift, cell, c->stream);
+    CKC(c, cudaGetLastError());
     const int one = 1, zero = 0;
     CKC(c, cudaMemcpy(c->ka.need_rebuild + cell, &one, sizeof(int), cudaMemcpyHostToDevice));
     CKC(c, cudaMemcpy(c->ka.status + cell, &zero, sizeof(int), cudaMemcpyHostToDevice));
@@ -866,7 +871,7 @@ int rcell_profile_kernels(rcell_ctx *c, int n_steps, double *ms_out) {
     };
     // coupling kernels once: re-apply the current F (Delta R = I), then the stress reduction
     CKC(c, cudaEventRecord(ev[0], c->stream));
-    rc_launch_deform_impl(c->d_F, c->d_H, c->d_Rprev, c->d_Q, c->d_R, c->d_F, c->d_dR, c->d_H0, c->d_Hf, c->d_Hif,
+    rc_launch_deform_impl(c->d_F, c->d_H, c->d_Rprev, c->d_Q, c->d_R, c->d_F, c->d_dR, c->d_H0, c->d_Hf, c->d_Hif, c->d_shift,
                           c->ka.status, c->ka.need_rebuild, c->d_nbins, c->d_bin_cap, c->ka.active, c->rlist, c->n_cells, c->stream);
     CKC(c, cudaEventRecord(ev[1], c->stream));
     rc_launch_remap(c->ka, c->d_dR, c->cur, c->n_tiles, c->stream);
@@ -884,7 +889,7 @@ int rcell_profile_kernels(rcell_ctx *c, int n_steps, double *ms_out) {
         CKC(c, cudaEventRecord(ev[0], c->stream));
         rc_launch_sort(c->kp, c->ka, c->cur, c->n_cells, c->stream);
         CKC(c, cudaEventRecord(ev[1], c->stream));
-        rc_launch_nlist(c->kp, c->ka, c->cur, c->n_tiles, c->stream);
+        rc_launch_nlist(c->kp, c->ka, c->cur, c->n_cells, c->stream);
         CKC(c, cudaEventRecord(ev[2], c->stream));
         if (c->kp.pot == RC_POT_SC) rc_launch_density(c->kp, c->ka, c->cur, c->n_tiles, c->tpa, stage_atoms(c), c->stream);
         CKC(c, cudaEventRecord(ev[3], c->stream));
