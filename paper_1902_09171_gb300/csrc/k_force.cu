@@ -94,8 +94,6 @@ __device__ __forceinline__ bool stage_records(float4 *dst, const float4 *src, in
     return false;
 }
 
-// Slots of a list group past the end of the list hold stale data: point them at
-// the group's first entry, which is always valid, so that they can be gathered.
 // List groups are read once per pass: loaded without allocating in L1, which
 // then keeps the neighbour records that the atoms of a tile share.
 __device__ __forceinline__ int4 ld_list(const int4 *p) {
@@ -119,60 +117,52 @@ inline unsigned pair_grid(const KParams &p) {
     return (unsigned)(((p.n_tiles + p.n_sm - 1) / p.n_sm) * p.n_sm);
 }
 
-__device__ __forceinline__ int4 clamp_group(int4 e, int left) {
-    if (left < 4) {
-        if (left < 2) e.y = e.x;
-        if (left < 3) e.z = e.x;
-        e.w = e.x;
-    }
-    return e;
-}
-
 // Displacements and pair evaluations of one list group (entries e, records
-// c0..c3, `left` entries of the list from this group on).  Warp-uniform fast
-// paths for full groups: all four entries of the image slot 0 (the central
-// image: x_j - x_i, the bits rc_disp gives for it) in every converged lane, or
-// one image slot per lane's group (the runs of a stencil bin): one shift-table
-// read and one x_i - sp per group instead of one per entry, the same arithmetic
-// as rc_disp.
+// c0..c3).  Warp-uniform fast paths: all four entries of the image slot 0 (the
+// central image: x_j - x_i, the bits rc_disp gives for it) in every converged
+// lane, or one image slot per lane's group (the runs of a stencil bin): one
+// shift-table read and one x_i - sp per group instead of one per entry, the same
+// arithmetic as rc_disp.  Null entries, which fill up a list's last group, have a
+// slot of their own whose displacement no cutoff reaches.
+//
+// fn is straight-line code: no branch on the cutoff,
+// which about two thirds of the lanes pass, so that the four evaluations
+// interleave.  The pair kernels are bound by the instructions they issue and the
+// L1 wavefronts of their gathers (0.7 of the issue slots, 0.6 of the L1 data
+// pipe on 320 000 beads); against a branch per entry and a check for the list's
+// end: force step without / with a sample 1956 / 2304 -> 1771 / 2117 us on
+// 10.24 M beads (lean walk), 56 / 61 -> 45 / 53 us on 160 000, density and force
+// of 128 000 copper atoms 71 + 80 -> 66 + 74 us.  (Packed FP32 arithmetic,
+// add / mul / fma.f32x2 on two neighbours, took another 2 to 6 % off the lean
+// walk but sums in another order; in the pipelined walk it spills.)
 template <class Fn>
-__device__ __forceinline__ void eval_group(const int4 &e, int left, const float4 &c0, const float4 &c1,
-                                           const float4 &c2, const float4 &c3, const float4 &xi, const ShiftTab &T,
-                                           Fn &&fn) {
+__device__ __forceinline__ void eval_group(const int4 &e, const float4 &c0, const float4 &c1, const float4 &c2,
+                                           const float4 &c3, const float4 &xi, const ShiftTab &T, Fn &&fn) {
     const unsigned s0 = (unsigned)e.x >> RC_IDX_BITS;
-    const bool one_slot =
-        left >= 4 && (((unsigned)(e.x ^ e.y) | (unsigned)(e.x ^ e.z) | (unsigned)(e.x ^ e.w)) >> RC_IDX_BITS) == 0;
     const unsigned am = __activemask();
     float3 d0, d1, d2, d3;
-    if (__all_sync(am, one_slot && s0 == RC_SLOT_CENTRAL)) {
+    if (__all_sync(am, ((unsigned)(e.x | e.y | e.z | e.w) >> RC_IDX_BITS) == RC_SLOT_CENTRAL)) {
         d0 = rc_disp_central(xi, c0);
         d1 = rc_disp_central(xi, c1);
         d2 = rc_disp_central(xi, c2);
         d3 = rc_disp_central(xi, c3);
-    } else if (__all_sync(am, one_slot)) {
+    } else if (__all_sync(am, (((unsigned)(e.x ^ e.y) | (unsigned)(e.x ^ e.z) | (unsigned)(e.x ^ e.w)) >> RC_IDX_BITS) == 0)) {
         const float4 sa = T.a[s0], sb = T.b[s0];
         const float4 xs = make_float4(xi.x - sb.x, xi.y - sb.y, xi.z - sb.z, sb.w);
         d0 = rc_disp_pre(c0, sa, xs);
         d1 = rc_disp_pre(c1, sa, xs);
         d2 = rc_disp_pre(c2, sa, xs);
         d3 = rc_disp_pre(c3, sa, xs);
-    } else {  // mixed image slots, or the list's last, partial group (whose missing
-              // entries repeat its first one: valid indices, results unused)
+    } else {
         d0 = rc_disp(xi, c0, T, s0);
         d1 = rc_disp(xi, c1, T, (unsigned)e.y >> RC_IDX_BITS);
         d2 = rc_disp(xi, c2, T, (unsigned)e.z >> RC_IDX_BITS);
         d3 = rc_disp(xi, c3, T, (unsigned)e.w >> RC_IDX_BITS);
     }
-    if (left >= 4) {
-        fn(c0, d0);
-        fn(c1, d1);
-        fn(c2, d2);
-        fn(c3, d3);
-    } else {
-        fn(c0, d0);
-        if (left > 1) fn(c1, d1);
-        if (left > 2) fn(c2, d2);
-    }
+    fn(c0, d0);
+    fn(c1, d1);
+    fn(c2, d2);
+    fn(c3, d3);
 }
 
 // Walk one atom's Verlet list (this lane's share: groups sub, sub+TPA, ... of
@@ -182,8 +172,8 @@ __device__ __forceinline__ void eval_group(const int4 &e, int left, const float4
 // the group after that are being loaded, so the gather latency overlaps the
 // pair arithmetic.  fn(xj, d) receives the neighbour's record and the exact
 // periodic displacement d = x_j(image) - x_i.
-// TPA == 0 is the lean walk: one lane per atom, one group at a time with no
-// pipelining -- fewer registers, so that more warps per SM hide the latency
+// TPA == 0 is the lean walk: one lane per atom, only the next group's entries
+// loaded ahead -- fewer registers, so that more warps per SM hide the latency
 // instead (the force kernel is compiled for 10 resident CTAs then, the density
 // kernel for 12), which pays when the batch has enough tiles to fill them.
 template <int TPA, class Src, class Fn>
@@ -191,21 +181,24 @@ __device__ __forceinline__ void for_each_neighbor(const int4 *__restrict__ nb4, 
                                                   const float4 &xi, const ShiftTab &T, Fn &&fn) {
     const int ng = (nn + 3) >> 2;
     if constexpr (TPA == 0) {
+        if (ng == 0) return;
+        int4 e = ld_list(nb4);
         for (int g = 0; g < ng; g++) {
             // the list streams from DRAM: ask L2 for the group after next now, so
             // that its load finds it there (no register holds it meanwhile)
-            if (g + 2 < ng) asm volatile("prefetch.global.L2 [%0];" ::"l"(nb4 + (size_t)(g + 2) * RC_TILE));
-            const int left = nn - 4 * g;
-            const int4 e = clamp_group(ld_list(nb4 + (size_t)g * RC_TILE), left);
+            if (g + 3 < ng) asm volatile("prefetch.global.L2 [%0];" ::"l"(nb4 + (size_t)(g + 3) * RC_TILE));
             const float4 c0 = src((unsigned)e.x & RC_IDX_MASK), c1 = src((unsigned)e.y & RC_IDX_MASK);
             const float4 c2 = src((unsigned)e.z & RC_IDX_MASK), c3 = src((unsigned)e.w & RC_IDX_MASK);
-            eval_group(e, left, c0, c1, c2, c3, xi, T, fn);
+            int4 en = e;
+            if (g + 1 < ng) en = ld_list(nb4 + (size_t)(g + 1) * RC_TILE);
+            eval_group(e, c0, c1, c2, c3, xi, T, fn);
+            e = en;
         }
         return;
     }
     int g = sub;
     if (g >= ng) return;
-    int4 e = clamp_group(ld_list(nb4 + (size_t)g * RC_TILE), nn - 4 * g);
+    int4 e = ld_list(nb4 + (size_t)g * RC_TILE);
     float4 c0 = src((unsigned)e.x & RC_IDX_MASK), c1 = src((unsigned)e.y & RC_IDX_MASK);
     float4 c2 = src((unsigned)e.z & RC_IDX_MASK), c3 = src((unsigned)e.w & RC_IDX_MASK);
     int gn = g + TPA;
@@ -216,53 +209,13 @@ __device__ __forceinline__ void for_each_neighbor(const int4 *__restrict__ nb4, 
         float4 n0 = c0, n1 = c1, n2 = c2, n3 = c3;
         int4 enn = en;
         if (gn < ng) {  // next stage: gather group gn, load the entries of group gnn
-            en = clamp_group(en, nn - 4 * gn);
             n0 = src((unsigned)en.x & RC_IDX_MASK);
             n1 = src((unsigned)en.y & RC_IDX_MASK);
             n2 = src((unsigned)en.z & RC_IDX_MASK);
             n3 = src((unsigned)en.w & RC_IDX_MASK);
             if (gnn < ng) enn = ld_list(nb4 + (size_t)gnn * RC_TILE);
         }
-        const int left = nn - 4 * g;
-        // Warp-uniform fast paths for full groups: all four entries of the image
-        // slot 0 (the central image: x_j - x_i, the bits rc_disp gives for it) in
-        // every converged lane, or one image slot per lane's group (the runs of a
-        // stencil bin): one shift-table read and one x_i - sp per group instead of
-        // one per entry, the same arithmetic as rc_disp.
-        const unsigned s0 = (unsigned)e.x >> RC_IDX_BITS;
-        const bool one_slot =
-            left >= 4 && (((unsigned)(e.x ^ e.y) | (unsigned)(e.x ^ e.z) | (unsigned)(e.x ^ e.w)) >> RC_IDX_BITS) == 0;
-        const unsigned am = __activemask();
-        float3 d0, d1, d2, d3;
-        if (__all_sync(am, one_slot && s0 == RC_SLOT_CENTRAL)) {
-            d0 = rc_disp_central(xi, c0);
-            d1 = rc_disp_central(xi, c1);
-            d2 = rc_disp_central(xi, c2);
-            d3 = rc_disp_central(xi, c3);
-        } else if (__all_sync(am, one_slot)) {
-            const float4 sa = T.a[s0], sb = T.b[s0];
-            const float4 xs = make_float4(xi.x - sb.x, xi.y - sb.y, xi.z - sb.z, sb.w);
-            d0 = rc_disp_pre(c0, sa, xs);
-            d1 = rc_disp_pre(c1, sa, xs);
-            d2 = rc_disp_pre(c2, sa, xs);
-            d3 = rc_disp_pre(c3, sa, xs);
-        } else {  // mixed image slots, or the list's last, partial group (whose missing
-                  // entries repeat its first one: valid indices, results unused)
-            d0 = rc_disp(xi, c0, T, s0);
-            d1 = rc_disp(xi, c1, T, (unsigned)e.y >> RC_IDX_BITS);
-            d2 = rc_disp(xi, c2, T, (unsigned)e.z >> RC_IDX_BITS);
-            d3 = rc_disp(xi, c3, T, (unsigned)e.w >> RC_IDX_BITS);
-        }
-        if (left >= 4) {
-            fn(c0, d0);
-            fn(c1, d1);
-            fn(c2, d2);
-            fn(c3, d3);
-        } else {
-            fn(c0, d0);
-            if (left > 1) fn(c1, d1);
-            if (left > 2) fn(c2, d2);
-        }
+        eval_group(e, c0, c1, c2, c3, xi, T, fn);
         if (gn >= ng) break;
         g = gn;
         gn = gnn;
@@ -273,6 +226,40 @@ __device__ __forceinline__ void for_each_neighbor(const int4 *__restrict__ nb4, 
         c2 = n2;
         c3 = n3;
     }
+}
+
+// rho + (a/r)^m of one neighbour (rho itself beyond the cutoff)
+template <bool M6>
+__device__ __forceinline__ float density_term(const KParams &p, const float3 &d, float rho) {
+    const float r2 = fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z));
+    const float ar2 = r2 < p.rc2 ? p.sigma * p.sigma * __fdividef(1.0f, r2) : 0.0f;
+    return M6 ? fmaf(ar2 * ar2, ar2, rho) : rho + (r2 < p.rc2 ? powf(ar2, 0.5f * p.sc_m) : 0.0f);
+}
+
+// dE/dr / r of one pair, and in e its energy in units of eps / 2 (SC) or 2 eps
+// (LJ); both zero beyond the cutoff, where 1 / r^2 counts as zero
+template <int POT, bool M6>
+__device__ __forceinline__ float pair_term(const KParams &p, const float4 &xi, const float4 &xj, const float3 &d, float &e) {
+    const float r2 = fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z));
+    const float ir2 = r2 < p.rc2 ? __fdividef(1.0f, r2) : 0.0f;
+    const float sr2 = p.sigma * p.sigma * ir2;
+    if (POT == RC_POT_SC) {
+        float arm, arn;
+        if (M6) {
+            arm = sr2 * sr2 * sr2;                     // (a/r)^6
+            arn = arm * sr2 * (p.sigma * rsqrtf(r2));  // (a/r)^9
+        } else {
+            arm = powf(sr2, 0.5f * p.sc_m);
+            arn = r2 < p.rc2 ? powf(sr2, 0.5f * p.sc_n) : 0.0f;
+        }
+        e = arn;
+        // eps / r^2 [ -n (a/r)^n + c m/2 (rho_i^-1/2 + rho_j^-1/2) (a/r)^m ]
+        return p.eps * ir2 * fmaf(0.5f * p.sc_c * p.sc_m * (xi.w + xj.w), arm, -p.sc_n * arn);
+    }
+    const float sr6 = sr2 * sr2 * sr2;
+    e = sr6 * (sr6 - 1.0f);
+    // -24 eps (2 (s/r)^12 - (s/r)^6) / r^2
+    return -(24.0f * p.eps) * ir2 * sr6 * (2.0f * sr6 - 1.0f);
 }
 
 // Sutton-Chen density pass: rho_i = sum_j (a/r_ij)^m over r < rc; writes
@@ -307,15 +294,7 @@ __global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), density_min_ctas(TPA))
         xi = X[g];
         const int nn = a.nnb[g];
         const int4 *__restrict__ nb = reinterpret_cast<const int4 *>(a.nbr) + (size_t)t * (p.max_nb / 4) * RC_TILE + at;
-        const float a2 = p.sigma * p.sigma, hm = 0.5f * p.sc_m;
-        const float rc2 = p.rc2;
-        auto body = [&](const float4 &, const float3 &d) {
-            const float r2 = fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z));
-            if (r2 < rc2) {
-                const float ar2 = a2 * __fdividef(1.0f, r2);
-                rho += M6 ? ar2 * ar2 * ar2 : powf(ar2, hm);
-            }
-        };
+        auto body = [&](const float4 &, const float3 &d) { rho = density_term<M6>(p, d, rho); };
         if (STG) for_each_neighbor<TPA>(nb, nn, sub, SharedSrc{s_cell, off}, xi, s_tab, body);
         else for_each_neighbor<TPA>(nb, nn, sub, GlobalSrc{X}, xi, s_tab, body);
     }
@@ -323,19 +302,29 @@ __global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), density_min_ctas(TPA))
     if (live && sub == 0) a.xr[g] = make_float4(xi.x, xi.y, xi.z, rho > 0.0f ? rsqrtf(rho) : 0.0f);
 }
 
-// Block reduction of NV per-atom float values into FP64, then one atomicAdd per
-// value into dst[0..NV).
+// Block reduction of NV <= 16 per-atom float values into FP64, then one
+// atomicAdd per value into dst[0..NV).  Within a warp the values are halved
+// together (lanes 16 .. 31 take over values 8 .. 15, and so on): 16 shuffles
+// instead of 5 NV, the same pairwise sums.
 template <int NV, int NT>
 __device__ __forceinline__ void block_reduce_add(float (&v)[NV], double *dst) {
-    __shared__ double s_part[NT / 32][NV];
+    static_assert(NV <= 16, "one value per lane pair");
+    __shared__ double s_part[NT / 32][16];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float w[16];
 #pragma unroll
-    for (int k = 0; k < NV; k++) {
-        float x = v[k];
+    for (int k = 0; k < 16; k++) w[k] = k < NV ? v[k < NV ? k : 0] : 0.0f;
 #pragma unroll
-        for (int d = 16; d >= 1; d >>= 1) x += __shfl_xor_sync(0xffffffffu, x, d);
-        if (lane == 0) s_part[warp][k] = (double)x;
+    for (int d = 16, h = 8; h >= 1; d >>= 1, h >>= 1) {
+        const bool up = lane & d;
+#pragma unroll
+        for (int k = 0; k < h; k++) {
+            const float mine = up ? w[k + h] : w[k], other = up ? w[k] : w[k + h];
+            w[k] = mine + __shfl_xor_sync(0xffffffffu, other, d);
+        }
     }
+    w[0] += __shfl_xor_sync(0xffffffffu, w[0], 1);
+    if ((lane & 1) == 0) s_part[warp][lane >> 1] = (double)w[0];  // lane bits 16 8 4 2: the value's bits 8 4 2 1
     __syncthreads();
     if (threadIdx.x < NV) {
         double s = 0.0;
@@ -348,22 +337,22 @@ __device__ __forceinline__ void block_reduce_add(float (&v)[NV], double *dst) {
 // Resident CTAs per SM the force kernel is compiled for at one lane per atom
 // (caps its registers at 65536 / (128 * RC_FORCE_MIN_CTAS)).  7 keeps a
 // 128 000-atom batch (1000 tiles) in one wave on 152 SMs; 1 leaves the
-// register count to the compiler.  The lean walk takes 10 (48 registers): on
-// the 80 000 tiles of a 10.24 M-bead batch, 12 (40 registers, with spills) ran
-// the force step 3 % and the sampling step 7 % slower, 8 and 9 (no spills)
-// 4-6 % and 1-3 % slower.
+// register count to the compiler.  The lean walk takes 10 (48 registers), with a
+// sample 8 (64 registers): on the 80 000 tiles of a 10.24 M-bead batch 12 (40
+// registers) ran 1.3 times as long, the force step at 9 and 8 1 and 4 % longer,
+// the sampling step at 7 and 6 7 % longer.
 #ifndef RC_FORCE_MIN_CTAS
 #define RC_FORCE_MIN_CTAS 7
 #endif
-constexpr int force_min_ctas(int tpa) {
-    return tpa == 0 ? 10 : (RC_FORCE_MIN_CTAS / tpa > 0 ? RC_FORCE_MIN_CTAS / tpa : 1);
+constexpr int force_min_ctas(int tpa, bool sample) {
+    return tpa == 0 ? (sample ? 8 : 10) : (RC_FORCE_MIN_CTAS / tpa > 0 ? RC_FORCE_MIN_CTAS / tpa : 1);
 }
 
 // SAMPLE: this launch records a stress sample (slot >= 0) or evaluates the
 // energy and virial (MODE_EVAL); without it the pair loop skips the virial and
 // energy terms, which only feed those records.
 template <int POT, int TPA, bool M6, bool STG, bool SAMPLE>
-__global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), force_min_ctas(TPA)) k_force(KParams p, KArrays a, int cur, int mode, int slot,
+__global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), force_min_ctas(TPA, SAMPLE)) k_force(KParams p, KArrays a, int cur, int mode, int slot,
                                                        int step_index) {
     extern __shared__ __align__(16) float4 s_cell[];
     rc_pdl_wait();
@@ -392,77 +381,27 @@ __global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), force_min_ctas(TPA)) k
         xi = XG[g];
         const int nn = a.nnb[g];
         const int4 *__restrict__ nb = reinterpret_cast<const int4 *>(a.nbr) + (size_t)t * (p.max_nb / 4) * RC_TILE + at;
-        if (POT == RC_POT_SC) {
-            const float a2 = p.sigma * p.sigma, hm = 0.5f * p.sc_m, hn = 0.5f * p.sc_n;
-            const float cm2 = 0.5f * p.sc_c * p.sc_m;
-            const float rc2 = p.rc2, eps = p.eps, sc_n = p.sc_n, sig = p.sigma;
-            auto body = [&](const float4 &xj, const float3 &d) {
-                const float dx = d.x, dy = d.y, dz = d.z;
-                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                if (r2 < rc2) {
-                    const float ir2 = __fdividef(1.0f, r2);
-                    const float ar2 = a2 * ir2;
-                    float arm, arn;
-                    if (M6) {
-                        arm = ar2 * ar2 * ar2;               // (a/r)^6
-                        arn = arm * ar2 * (sig * rsqrtf(r2));  // (a/r)^9
-                    } else {
-                        arm = powf(ar2, hm);
-                        arn = powf(ar2, hn);
-                    }
-                    // dE/dr / r = eps / r^2 [ -n (a/r)^n + c m/2 (rho_i^-1/2 + rho_j^-1/2) (a/r)^m ]
-                    const float gr = eps * ir2 * fmaf(cm2 * (xi.w + xj.w), arm, -sc_n * arn);
-                    const float gx = gr * dx, gy = gr * dy, gz = gr * dz;
-                    fx += gx;
-                    fy += gy;
-                    fz += gz;
-                    if (SAMPLE) {  // scaled once per atom after the walk: W by -1/2, pe by eps/2
-                        w0 = fmaf(gx, dx, w0);
-                        w1 = fmaf(gy, dy, w1);
-                        w2 = fmaf(gz, dz, w2);
-                        w3 = fmaf(gx, dy, w3);
-                        w4 = fmaf(gx, dz, w4);
-                        w5 = fmaf(gy, dz, w5);
-                        pe += arn;
-                    }
-                }
-            };
-            if (STG) for_each_neighbor<TPA>(nb, nn, sub, SharedSrc{s_cell, off}, xi, s_tab, body);
-            else for_each_neighbor<TPA>(nb, nn, sub, GlobalSrc{XG}, xi, s_tab, body);
-            if (SAMPLE) pe *= 0.5f * eps;
-        } else {
-            const float s2 = p.sigma * p.sigma;
-            const float c24 = 24.0f * p.eps, c2 = 2.0f * p.eps;
-            const float rc2 = p.rc2;
-            auto body = [&](const float4 &, const float3 &d) {
-                const float dx = d.x, dy = d.y, dz = d.z;
-                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                if (r2 < rc2) {
-                    const float ir2 = __fdividef(1.0f, r2);
-                    const float sr2 = s2 * ir2;
-                    const float sr6 = sr2 * sr2 * sr2;
-                    // dU/dr / r = -24 eps (2 (s/r)^12 - (s/r)^6) / r^2
-                    const float gr = -c24 * ir2 * sr6 * (2.0f * sr6 - 1.0f);
-                    const float gx = gr * dx, gy = gr * dy, gz = gr * dz;
-                    fx += gx;
-                    fy += gy;
-                    fz += gz;
-                    if (SAMPLE) {  // scaled once per atom after the walk: W by -1/2, pe by 2 eps
-                        w0 = fmaf(gx, dx, w0);
-                        w1 = fmaf(gy, dy, w1);
-                        w2 = fmaf(gz, dz, w2);
-                        w3 = fmaf(gx, dy, w3);
-                        w4 = fmaf(gx, dz, w4);
-                        w5 = fmaf(gy, dz, w5);
-                        pe = fmaf(sr6, sr6 - 1.0f, pe);  // 1/2 * 4 eps (sr12 - sr6) / (2 eps)
-                    }
-                }
-            };
-            if (STG) for_each_neighbor<TPA>(nb, nn, sub, SharedSrc{s_cell, off}, xi, s_tab, body);
-            else for_each_neighbor<TPA>(nb, nn, sub, GlobalSrc{XG}, xi, s_tab, body);
-            if (SAMPLE) pe *= c2;
-        }
+        auto body = [&](const float4 &xj, const float3 &d) {
+            float e;
+            const float gr = pair_term<POT, M6>(p, xi, xj, d, e);
+            const float gx = gr * d.x, gy = gr * d.y, gz = gr * d.z;
+            fx += gx;
+            fy += gy;
+            fz += gz;
+            if (SAMPLE) {  // scaled once per atom after the walk
+                w0 = fmaf(gx, d.x, w0);
+                w1 = fmaf(gy, d.y, w1);
+                w2 = fmaf(gz, d.z, w2);
+                w3 = fmaf(gx, d.y, w3);
+                w4 = fmaf(gx, d.z, w4);
+                w5 = fmaf(gy, d.z, w5);
+                pe += e;
+            }
+        };
+        if (STG) for_each_neighbor<TPA>(nb, nn, sub, SharedSrc{s_cell, off}, xi, s_tab, body);
+        else for_each_neighbor<TPA>(nb, nn, sub, GlobalSrc{XG}, xi, s_tab, body);
         if (SAMPLE) {
+            pe *= POT == RC_POT_SC ? 0.5f * p.eps : 2.0f * p.eps;
             w0 *= -0.5f;
             w1 *= -0.5f;
             w2 *= -0.5f;
@@ -634,35 +573,10 @@ __global__ void __launch_bounds__(RC_TILE) k_static_pk1(KParams p, KArrays a, in
         const int nn = a.nnb[g];
         const int4 *__restrict__ nb =
             reinterpret_cast<const int4 *>(a.nbr) + (size_t)t * (p.max_nb / 4) * RC_TILE + threadIdx.x;
-        const float rc2 = p.rc2;
-        if (POT == RC_POT_SC) {
-            const float a2 = p.sigma * p.sigma, hm = 0.5f * p.sc_m, hn = 0.5f * p.sc_n;
-            const float cm2 = 0.5f * p.sc_c * p.sc_m, eps = p.eps, sc_n = p.sc_n, sig = p.sigma;
-            for_each_neighbor<1>(nb, nn, 0, GlobalSrc{XG}, xi, s_tab, [&](const float4 &xj, const float3 &d) {
-                const float r2 = fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z));
-                if (r2 < rc2) {
-                    const float ir2 = __fdividef(1.0f, r2), ar2 = a2 * ir2;
-                    float arm, arn;
-                    if (M6) {
-                        arm = ar2 * ar2 * ar2;
-                        arn = arm * ar2 * (sig * rsqrtf(r2));
-                    } else {
-                        arm = powf(ar2, hm);
-                        arn = powf(ar2, hn);
-                    }
-                    add(eps * ir2 * fmaf(cm2 * (xi.w + xj.w), arm, -sc_n * arn), d);
-                }
-            });
-        } else {
-            const float s2 = p.sigma * p.sigma, c24 = 24.0f * p.eps;
-            for_each_neighbor<1>(nb, nn, 0, GlobalSrc{XG}, xi, s_tab, [&](const float4 &, const float3 &d) {
-                const float r2 = fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z));
-                if (r2 < rc2) {
-                    const float ir2 = __fdividef(1.0f, r2), sr2 = s2 * ir2, sr6 = sr2 * sr2 * sr2;
-                    add(-c24 * ir2 * sr6 * (2.0f * sr6 - 1.0f), d);
-                }
-            });
-        }
+        for_each_neighbor<1>(nb, nn, 0, GlobalSrc{XG}, xi, s_tab, [&](const float4 &xj, const float3 &d) {
+            float e;
+            add(pair_term<POT, M6>(p, xi, xj, d, e), d);
+        });
         if (POT == RC_POT_KG) {
             const int4 pr = a.partner[g];
             const int q[4] = {pr.x, pr.y, pr.z, pr.w};
