@@ -193,7 +193,11 @@ int rcell_clear_status(rcell_ctx *ctx);
  *                      walking the list software-pipelined (the next group's
  *                      gathers in flight while a group is evaluated); 0 = one
  *                      lane per atom with a plain walk compiled for more
- *                      resident warps per SM (pays on large batches)
+ *                      resident warps per SM (pays on large batches).
+ *                      With 0 and 1, batches (or active cells, where the host
+ *                      gave the mask) of few atoms are walked by sixteen lanes
+ *                      per atom that add in the same order: the same results
+ *                      bit for bit
  *   use_graphs       : 0/1, capture rcell_run into CUDA graphs
  * All settings give the same results up to summation order. */
 int rcell_set_tuning(rcell_ctx *ctx, int threads_per_atom, int use_graphs);

@@ -108,10 +108,18 @@ __device__ __forceinline__ int4 ld_list(const int4 *p) {
 // SM count S, and block b takes tile (b mod S) R + b / S: blocks b, b + S,
 // b + 2S, ... -- those that the first wave deals to one SM -- get consecutive
 // tiles, the spatial neighbours of one r-cell, whose shared neighbour records
-// then stay in that SM's L1.  Blocks past the last tile return at once.
-__device__ __forceinline__ int tile_of_block(int n_sm) {
-    const int R = (int)gridDim.x / n_sm;
-    return (int)(blockIdx.x % n_sm) * R + (int)(blockIdx.x / n_sm);
+// then stay in that SM's L1.  Blocks past the last tile return at once (-1).
+// When cells are switched off, the same over the tiles of the others: by tile
+// number, three active cells of 32 x 4000 atoms ran on 14 SMs and took as long
+// as all 32.
+__device__ __forceinline__ int tile_of_block(const KParams &p, const KArrays &a) {
+    const int at = (int)(blockIdx.x % p.n_sm), row = (int)(blockIdx.x / p.n_sm);
+    if (!p.masked) {
+        const int t = at * ((int)gridDim.x / p.n_sm) + row;
+        return t < p.n_tiles ? t : -1;
+    }
+    const int n = *a.n_act, rows = (n + p.n_sm - 1) / p.n_sm, k = at * rows + row;
+    return row < rows && k < n ? a.act_tiles[k] : -1;
 }
 inline unsigned pair_grid(const KParams &p) {
     return (unsigned)(((p.n_tiles + p.n_sm - 1) / p.n_sm) * p.n_sm);
@@ -228,12 +236,17 @@ __device__ __forceinline__ void for_each_neighbor(const int4 *__restrict__ nb4, 
     }
 }
 
-// rho + (a/r)^m of one neighbour (rho itself beyond the cutoff)
+// One neighbour's part in rho, zero beyond the cutoff: (a/r)^2 for m = 6, else
+// (a/r)^m, and the sum with it
 template <bool M6>
-__device__ __forceinline__ float density_term(const KParams &p, const float3 &d, float rho) {
+__device__ __forceinline__ float density_term(const KParams &p, const float3 &d) {
     const float r2 = fmaf(d.x, d.x, fmaf(d.y, d.y, d.z * d.z));
     const float ar2 = r2 < p.rc2 ? p.sigma * p.sigma * __fdividef(1.0f, r2) : 0.0f;
-    return M6 ? fmaf(ar2 * ar2, ar2, rho) : rho + (r2 < p.rc2 ? powf(ar2, 0.5f * p.sc_m) : 0.0f);
+    return M6 || !(r2 < p.rc2) ? ar2 : powf(ar2, 0.5f * p.sc_m);
+}
+template <bool M6>
+__device__ __forceinline__ float density_sum(float rho, float q) {
+    return M6 ? fmaf(q * q, q, rho) : __fadd_rn(rho, q);
 }
 
 // dE/dr / r of one pair, and in e its energy in units of eps / 2 (SC) or 2 eps
@@ -274,8 +287,8 @@ __global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), density_min_ctas(TPA))
     extern __shared__ __align__(16) float4 s_cell[];
     rc_pdl_wait();
     rc_pdl_trigger();
-    const int t = tile_of_block(p.n_sm);
-    if (t >= p.n_tiles) return;
+    const int t = tile_of_block(p, a);
+    if (t < 0) return;
     const int c = a.tile_cell[t];
     if (a.status[c] != 0 || !a.active[c]) return;
     __shared__ ShiftTab s_tab;
@@ -294,7 +307,7 @@ __global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), density_min_ctas(TPA))
         xi = X[g];
         const int nn = a.nnb[g];
         const int4 *__restrict__ nb = reinterpret_cast<const int4 *>(a.nbr) + (size_t)t * (p.max_nb / 4) * RC_TILE + at;
-        auto body = [&](const float4 &, const float3 &d) { rho = density_term<M6>(p, d, rho); };
+        auto body = [&](const float4 &, const float3 &d) { rho = density_sum<M6>(rho, density_term<M6>(p, d)); };
         if (STG) for_each_neighbor<TPA>(nb, nn, sub, SharedSrc{s_cell, off}, xi, s_tab, body);
         else for_each_neighbor<TPA>(nb, nn, sub, GlobalSrc{X}, xi, s_tab, body);
     }
@@ -325,7 +338,8 @@ __device__ __forceinline__ void block_reduce_add(float (&v)[NV], double *dst) {
     }
     w[0] += __shfl_xor_sync(0xffffffffu, w[0], 1);
     if ((lane & 1) == 0) s_part[warp][lane >> 1] = (double)w[0];  // lane bits 16 8 4 2: the value's bits 8 4 2 1
-    __syncthreads();
+    if (NT == 32) __syncwarp();
+    else __syncthreads();
     if (threadIdx.x < NV) {
         double s = 0.0;
 #pragma unroll
@@ -334,96 +348,15 @@ __device__ __forceinline__ void block_reduce_add(float (&v)[NV], double *dst) {
     }
 }
 
-// Resident CTAs per SM the force kernel is compiled for at one lane per atom
-// (caps its registers at 65536 / (128 * RC_FORCE_MIN_CTAS)).  7 keeps a
-// 128 000-atom batch (1000 tiles) in one wave on 152 SMs; 1 leaves the
-// register count to the compiler.  The lean walk takes 10 (48 registers), with a
-// sample 8 (64 registers): on the 80 000 tiles of a 10.24 M-bead batch 12 (40
-// registers) ran 1.3 times as long, the force step at 9 and 8 1 and 4 % longer,
-// the sampling step at 7 and 6 7 % longer.
-#ifndef RC_FORCE_MIN_CTAS
-#define RC_FORCE_MIN_CTAS 7
-#endif
-constexpr int force_min_ctas(int tpa, bool sample) {
-    return tpa == 0 ? (sample ? 8 : 10) : (RC_FORCE_MIN_CTAS / tpa > 0 ? RC_FORCE_MIN_CTAS / tpa : 1);
-}
-
-// SAMPLE: this launch records a stress sample (slot >= 0) or evaluates the
-// energy and virial (MODE_EVAL); without it the pair loop skips the virial and
-// energy terms, which only feed those records.
-template <int POT, int TPA, bool M6, bool STG, bool SAMPLE>
-__global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), force_min_ctas(TPA, SAMPLE)) k_force(KParams p, KArrays a, int cur, int mode, int slot,
-                                                       int step_index) {
-    extern __shared__ __align__(16) float4 s_cell[];
-    rc_pdl_wait();
-    rc_pdl_trigger();
-    const int t = tile_of_block(p.n_sm);
-    if (t >= p.n_tiles) return;
-    const int c = a.tile_cell[t];
-    if (a.status[c] != 0 || !a.active[c]) return;
-    __shared__ ShiftTab s_tab;
-    rc_load_shifts(s_tab, a.shift, c);
-
-    const int at = threadIdx.x / lanes_of(TPA), sub = threadIdx.x % lanes_of(TPA);
-    const int n = a.cell_n[c], off = a.cell_off[c];
-    const int li = (t - a.cell_tile0[c]) * RC_TILE + at;
-    const bool live = li < n;
-    const int g = off + li;
-    const float4 *__restrict__ X = cur ? a.x1 : a.x0;
-    const float4 *__restrict__ XG = (POT == RC_POT_SC) ? a.xr : X;  // gathered array
-    if (STG && !stage_records(s_cell, XG + off, n, a.status, c, p.wait_polls)) return;
-
-    float fx = 0.f, fy = 0.f, fz = 0.f;
-    float w0 = 0.f, w1 = 0.f, w2 = 0.f, w3 = 0.f, w4 = 0.f, w5 = 0.f;  // xx yy zz xy xz yz
-    float pe = 0.f;
-    float4 xi = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (live) {
-        xi = XG[g];
-        const int nn = a.nnb[g];
-        const int4 *__restrict__ nb = reinterpret_cast<const int4 *>(a.nbr) + (size_t)t * (p.max_nb / 4) * RC_TILE + at;
-        auto body = [&](const float4 &xj, const float3 &d) {
-            float e;
-            const float gr = pair_term<POT, M6>(p, xi, xj, d, e);
-            const float gx = gr * d.x, gy = gr * d.y, gz = gr * d.z;
-            fx += gx;
-            fy += gy;
-            fz += gz;
-            if (SAMPLE) {  // scaled once per atom after the walk
-                w0 = fmaf(gx, d.x, w0);
-                w1 = fmaf(gy, d.y, w1);
-                w2 = fmaf(gz, d.z, w2);
-                w3 = fmaf(gx, d.y, w3);
-                w4 = fmaf(gx, d.z, w4);
-                w5 = fmaf(gy, d.z, w5);
-                pe += e;
-            }
-        };
-        if (STG) for_each_neighbor<TPA>(nb, nn, sub, SharedSrc{s_cell, off}, xi, s_tab, body);
-        else for_each_neighbor<TPA>(nb, nn, sub, GlobalSrc{XG}, xi, s_tab, body);
-        if (SAMPLE) {
-            pe *= POT == RC_POT_SC ? 0.5f * p.eps : 2.0f * p.eps;
-            w0 *= -0.5f;
-            w1 *= -0.5f;
-            w2 *= -0.5f;
-            w3 *= -0.5f;
-            w4 *= -0.5f;
-            w5 *= -0.5f;
-        }
-    }
-    fx = sub_sum<TPA>(fx);
-    fy = sub_sum<TPA>(fy);
-    fz = sub_sum<TPA>(fz);
-    if (SAMPLE) {
-        w0 = sub_sum<TPA>(w0);
-        w1 = sub_sum<TPA>(w1);
-        w2 = sub_sum<TPA>(w2);
-        w3 = sub_sum<TPA>(w3);
-        w4 = sub_sum<TPA>(w4);
-        w5 = sub_sum<TPA>(w5);
-        pe = sub_sum<TPA>(pe);
-    }
-    const bool own = live && sub == 0;
-
+// What follows the sums over an atom's neighbours (force f, virial w, energy pe):
+// the embedding energy, the chain bonds, and the integration step or, in
+// MODE_EVAL, the result.  One thread per atom (own), NT threads per block;
+// bonded[k] is the record of atom k of the cell.
+template <int POT, int NT>
+__device__ __forceinline__ void finish_atom(const KParams &p, const KArrays &a, int cur, int mode, int slot, int step_index,
+                                            int c, int g, bool own, const float4 &xi, const ShiftTab &s_tab,
+                                            const float4 *bonded, float fx, float fy, float fz, float w0, float w1,
+                                            float w2, float w3, float w4, float w5, float pe) {
     if (own && POT == RC_POT_SC && xi.w > 0.0f) pe -= p.eps * p.sc_c / xi.w;  // embedding -eps c sqrt(rho_i)
 
     if (own && POT == RC_POT_KG) {
@@ -435,7 +368,7 @@ __global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), force_min_ctas(TPA, SA
 #pragma unroll
         for (int b = 0; b < RC_MAX_BONDS; b++) {
             if (q[b] < 0) continue;
-            const float4 xj = STG ? s_cell[q[b]] : X[off + q[b]];
+            const float4 xj = bonded[q[b]];
             // minimum image: pick the integer shift from fractional coordinates, then
             // form the displacement through the exact shift table
             const float ex = xj.x - xi.x, ey = xj.y - xi.y, ez = xj.z - xi.z;
@@ -478,7 +411,7 @@ __global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), force_min_ctas(TPA, SA
         if (own) a.f[g] = make_float4(fx, fy, fz, pe);
         float v[7] = {own ? pe : 0.f, own ? w0 : 0.f, own ? w1 : 0.f, own ? w2 : 0.f,
                       own ? w3 : 0.f, own ? w4 : 0.f, own ? w5 : 0.f};
-        block_reduce_add<7, RC_TILE * lanes_of(TPA)>(v, a.eval_acc + 8 * c);
+        block_reduce_add<7, NT>(v, a.eval_acc + 8 * c);
         return;
     }
 
@@ -536,8 +469,264 @@ __global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), force_min_ctas(TPA, SA
         float v[13] = {kxx, kyy, kzz, kxy, kxz, kyz,
                        own ? w0 : 0.f, own ? w1 : 0.f, own ? w2 : 0.f, own ? w3 : 0.f, own ? w4 : 0.f, own ? w5 : 0.f,
                        own ? pe : 0.f};
-        block_reduce_add<13, RC_TILE * lanes_of(TPA)>(v, a.series + ((size_t)c * a.series_cap + slot) * RC_SAMPLE_W);
+        block_reduce_add<13, NT>(v, a.series + ((size_t)c * a.series_cap + slot) * RC_SAMPLE_W);
     }
+}
+
+// Resident CTAs per SM the force kernel is compiled for at one lane per atom
+// (caps its registers at 65536 / (128 * RC_FORCE_MIN_CTAS)).  7 keeps a
+// 128 000-atom batch (1000 tiles) in one wave on 152 SMs; 1 leaves the
+// register count to the compiler.  The lean walk takes 10 (48 registers), with a
+// sample 8 (64 registers): on the 80 000 tiles of a 10.24 M-bead batch 12 (40
+// registers) ran 1.3 times as long, the force step at 9 and 8 1 and 4 % longer,
+// the sampling step at 7 and 6 7 % longer.
+#ifndef RC_FORCE_MIN_CTAS
+#define RC_FORCE_MIN_CTAS 7
+#endif
+constexpr int force_min_ctas(int tpa, bool sample) {
+    return tpa == 0 ? (sample ? 8 : 10) : (RC_FORCE_MIN_CTAS / tpa > 0 ? RC_FORCE_MIN_CTAS / tpa : 1);
+}
+
+// SAMPLE: this launch records a stress sample (slot >= 0) or evaluates the
+// energy and virial (MODE_EVAL); without it the pair loop skips the virial and
+// energy terms, which only feed those records.
+template <int POT, int TPA, bool M6, bool STG, bool SAMPLE>
+__global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), force_min_ctas(TPA, SAMPLE)) k_force(KParams p, KArrays a, int cur, int mode, int slot,
+                                                       int step_index) {
+    extern __shared__ __align__(16) float4 s_cell[];
+    rc_pdl_wait();
+    rc_pdl_trigger();
+    const int t = tile_of_block(p, a);
+    if (t < 0) return;
+    const int c = a.tile_cell[t];
+    if (a.status[c] != 0 || !a.active[c]) return;
+    __shared__ ShiftTab s_tab;
+    rc_load_shifts(s_tab, a.shift, c);
+
+    const int at = threadIdx.x / lanes_of(TPA), sub = threadIdx.x % lanes_of(TPA);
+    const int n = a.cell_n[c], off = a.cell_off[c];
+    const int li = (t - a.cell_tile0[c]) * RC_TILE + at;
+    const bool live = li < n;
+    const int g = off + li;
+    const float4 *__restrict__ X = cur ? a.x1 : a.x0;
+    const float4 *__restrict__ XG = (POT == RC_POT_SC) ? a.xr : X;  // gathered array
+    if (STG && !stage_records(s_cell, XG + off, n, a.status, c, p.wait_polls)) return;
+
+    float fx = 0.f, fy = 0.f, fz = 0.f;
+    float w0 = 0.f, w1 = 0.f, w2 = 0.f, w3 = 0.f, w4 = 0.f, w5 = 0.f;  // xx yy zz xy xz yz
+    float pe = 0.f;
+    float4 xi = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (live) {
+        xi = XG[g];
+        const int nn = a.nnb[g];
+        const int4 *__restrict__ nb = reinterpret_cast<const int4 *>(a.nbr) + (size_t)t * (p.max_nb / 4) * RC_TILE + at;
+        auto body = [&](const float4 &xj, const float3 &d) {
+            float e;
+            const float gr = pair_term<POT, M6>(p, xi, xj, d, e);
+            if (!SAMPLE) {
+                fx = fmaf(gr, d.x, fx);
+                fy = fmaf(gr, d.y, fy);
+                fz = fmaf(gr, d.z, fz);
+            } else {  // w, pe: scaled once per atom after the walk
+                const float gx = gr * d.x, gy = gr * d.y, gz = gr * d.z;
+                fx = __fadd_rn(fx, gx);
+                fy = __fadd_rn(fy, gy);
+                fz = __fadd_rn(fz, gz);
+                w0 = fmaf(gx, d.x, w0);
+                w1 = fmaf(gy, d.y, w1);
+                w2 = fmaf(gz, d.z, w2);
+                w3 = fmaf(gx, d.y, w3);
+                w4 = fmaf(gx, d.z, w4);
+                w5 = fmaf(gy, d.z, w5);
+                pe = __fadd_rn(pe, e);
+            }
+        };
+        if (STG) for_each_neighbor<TPA>(nb, nn, sub, SharedSrc{s_cell, off}, xi, s_tab, body);
+        else for_each_neighbor<TPA>(nb, nn, sub, GlobalSrc{XG}, xi, s_tab, body);
+        if (SAMPLE) {
+            pe *= POT == RC_POT_SC ? 0.5f * p.eps : 2.0f * p.eps;
+            w0 *= -0.5f;
+            w1 *= -0.5f;
+            w2 *= -0.5f;
+            w3 *= -0.5f;
+            w4 *= -0.5f;
+            w5 *= -0.5f;
+        }
+    }
+    fx = sub_sum<TPA>(fx);
+    fy = sub_sum<TPA>(fy);
+    fz = sub_sum<TPA>(fz);
+    if (SAMPLE) {
+        w0 = sub_sum<TPA>(w0);
+        w1 = sub_sum<TPA>(w1);
+        w2 = sub_sum<TPA>(w2);
+        w3 = sub_sum<TPA>(w3);
+        w4 = sub_sum<TPA>(w4);
+        w5 = sub_sum<TPA>(w5);
+        pe = sub_sum<TPA>(pe);
+    }
+    const float4 *bonded = STG ? s_cell : X + off;
+    finish_atom<POT, RC_TILE * lanes_of(TPA)>(p, a, cur, mode, slot, step_index, c, g, live && sub == 0, xi, s_tab, bonded,
+                                              fx, fy, fz, w0, w1, w2, w3, w4, w5, pe);
+}
+
+// ---------------------------------------------------------------------------
+// The cooperative walk, for batches too small to fill the chip: sixteen lanes
+// share an atom, in CTAs of 32 atoms (a quarter of a tile).  Each lane evaluates
+// one list entry of a round of sixteen and leaves the displacement and dE/dr / r
+// in shared memory; then lane r < 10 adds component r of force, virial (xx yy zz
+// xy xz yz) and energy over the sixteen entries in list order, four at a time per
+// shared load, so that every sum has the bits of the one-lane walk and a batch
+// can change between the two at any step.  The last round's missing entries are
+// null entries.  The first warp then finishes the 32 atoms as k_force does.
+// One lane per atom is a chain of one gather latency per group of four entries
+// (236 entries in copper at skin 1.5 A) however few tiles there are: the 256-atom
+// LJ cell's step takes 10.7 us instead of 16.3, that of three active 4000-atom
+// copper cells of 32 takes 41 us instead of 93.
+// ---------------------------------------------------------------------------
+constexpr int COOP_LANES = 16, COOP_ATOMS = 32, COOP_THREADS = COOP_LANES * COOP_ATOMS;
+constexpr int COOP_PER_TILE = RC_TILE / COOP_ATOMS, COOP_ROW = COOP_LANES + 4, COOP_COMP = COOP_ATOMS * COOP_ROW + 4;
+
+// this CTA's tile, or -1
+__device__ __forceinline__ int coop_tile(const KParams &p, const KArrays &a) {
+    const int k = (int)(blockIdx.x / COOP_PER_TILE);
+    if (!p.masked) return k < p.n_tiles ? k : -1;
+    return k < *a.n_act ? a.act_tiles[k] : -1;
+}
+
+// The rounds of one atom's list (entry k at nb[(k / 4) 4 TILE + k % 4]; both
+// atoms of a warp take the same number): eval(xj, d) on this lane's entry, then
+// sum() with all sixteen results in place.  The next round's gathers are in
+// flight meanwhile.
+template <class Eval, class Sum>
+__device__ __forceinline__ void coop_walk(const int *__restrict__ nb, int nn, unsigned self, const float4 *__restrict__ X,
+                                          const float4 &xi, const ShiftTab &T, Eval &&eval, Sum &&sum) {
+    const int l = threadIdx.x % COOP_LANES;
+    int rounds = (nn + COOP_LANES - 1) / COOP_LANES;
+    rounds = max(rounds, __shfl_xor_sync(0xffffffffu, rounds, COOP_LANES));
+    const auto entry = [&](int r) {
+        const int k = r * COOP_LANES + l;
+        return k < nn ? (unsigned)__ldg(nb + (size_t)(k >> 2) * (4 * RC_TILE) + (k & 3)) : self | RC_SLOT_NULL << RC_IDX_BITS;
+    };
+    unsigned e = entry(0), en = entry(1);
+    float4 xj = __ldg(X + (e & RC_IDX_MASK));
+    for (int r = 0; r < rounds; r++) {
+        const float4 xn = __ldg(X + (en & RC_IDX_MASK));
+        const unsigned enn = entry(r + 2);
+        const unsigned slot = e >> RC_IDX_BITS;
+        eval(xj, __all_sync(0xffffffffu, slot == RC_SLOT_CENTRAL) ? rc_disp_central(xi, xj) : rc_disp(xi, xj, T, slot));
+        __syncwarp();
+        sum();
+        __syncwarp();
+        e = en;
+        en = enn;
+        xj = xn;
+    }
+}
+
+template <bool M6, int CTAS>
+__global__ void __launch_bounds__(COOP_THREADS, CTAS) k_density_coop(KParams p, KArrays a, int cur) {
+    __shared__ ShiftTab s_tab;
+    __shared__ __align__(16) float s_q[COOP_ATOMS][COOP_ROW];
+    rc_pdl_wait();
+    rc_pdl_trigger();
+    const int t = coop_tile(p, a);
+    if (t < 0) return;
+    const int c = a.tile_cell[t];
+    if (a.status[c] != 0 || !a.active[c]) return;
+    rc_load_shifts(s_tab, a.shift, c);
+    const int at = threadIdx.x / COOP_LANES, l = threadIdx.x % COOP_LANES;
+    const int in_tile = (int)(blockIdx.x % COOP_PER_TILE) * COOP_ATOMS + at;
+    const int li = (t - a.cell_tile0[c]) * RC_TILE + in_tile, n = a.cell_n[c], off = a.cell_off[c];
+    const int g = off + min(li, n - 1);
+    const float4 *__restrict__ X = cur ? a.x1 : a.x0;
+    const float4 xi = X[g];
+    float rho = 0.0f;
+    coop_walk(a.nbr + (size_t)t * p.max_nb * RC_TILE + 4 * in_tile, li < n ? a.nnb[g] : 0, (unsigned)g, X, xi, s_tab,
+              [&](const float4 &, const float3 &d) { s_q[at][l] = density_term<M6>(p, d); },
+              [&] {
+#pragma unroll
+                  for (int k = 0; k < COOP_LANES; k += 4) {  // (every lane; lane 0's is used)
+                      const float4 q = *reinterpret_cast<const float4 *>(&s_q[at][k]);
+                      rho = density_sum<M6>(rho, q.x);
+                      rho = density_sum<M6>(rho, q.y);
+                      rho = density_sum<M6>(rho, q.z);
+                      rho = density_sum<M6>(rho, q.w);
+                  }
+              });
+    if (li < n && l == 0) a.xr[g] = make_float4(xi.x, xi.y, xi.z, rho > 0.0f ? rsqrtf(rho) : 0.0f);
+}
+
+template <int POT, bool M6, bool SAMPLE, int CTAS>
+__global__ void __launch_bounds__(COOP_THREADS, CTAS) k_force_coop(KParams p, KArrays a, int cur, int mode, int slot, int step_index) {
+    __shared__ ShiftTab s_tab;
+    __shared__ __align__(16) float s_pair[SAMPLE ? 5 : 4][COOP_COMP];  // d (3), dE/dr / r, energy: [atom][entry]
+    __shared__ float s_sum[COOP_ATOMS][11];
+    rc_pdl_wait();
+    rc_pdl_trigger();
+    const int t = coop_tile(p, a);
+    if (t < 0) return;
+    const int c = a.tile_cell[t];
+    if (a.status[c] != 0 || !a.active[c]) return;
+    rc_load_shifts(s_tab, a.shift, c);
+    const int at = threadIdx.x / COOP_LANES, l = threadIdx.x % COOP_LANES;
+    const int n = a.cell_n[c], off = a.cell_off[c];
+    const int in0 = (int)(blockIdx.x % COOP_PER_TILE) * COOP_ATOMS, li0 = (t - a.cell_tile0[c]) * RC_TILE + in0;
+    const float4 *__restrict__ X = cur ? a.x1 : a.x0;
+    const float4 *__restrict__ XG = (POT == RC_POT_SC) ? a.xr : X;
+    {
+        const int li = li0 + at, g = off + min(li, n - 1);
+        const float4 xi = XG[g];
+        // lane r adds force component r, virial component r - 3 = (ia, ib), or the energy
+        const int ia = l < 3 ? l : (l < 6 ? l - 3 : (l < 8 ? 0 : 1)), ib = l < 6 ? l - 3 : (l == 6 ? 1 : 2);
+        const bool f = l < 3, w = l >= 3 && l < 9;
+        const int row = at * COOP_ROW;
+        const float *pa = &s_pair[l == 9 && SAMPLE ? 4 : ia][row], *pb = &s_pair[w ? ib : 0][row], *pg = &s_pair[3][row];
+        float acc = 0.0f;
+        const auto one = [&](float gr, float da, float db) {
+            const float v = gr * da;
+            if (!SAMPLE) acc = fmaf(gr, da, acc);
+            else acc = w ? fmaf(v, db, acc) : __fadd_rn(acc, f ? v : da);
+        };
+        coop_walk(a.nbr + (size_t)t * p.max_nb * RC_TILE + 4 * (in0 + at), li < n ? a.nnb[g] : 0, (unsigned)g, XG, xi, s_tab,
+                  [&](const float4 &xj, const float3 &d) {
+                      float e;
+                      const float gr = pair_term<POT, M6>(p, xi, xj, d, e);
+                      s_pair[0][row + l] = d.x;
+                      s_pair[1][row + l] = d.y;
+                      s_pair[2][row + l] = d.z;
+                      s_pair[3][row + l] = gr;
+                      if (SAMPLE) s_pair[SAMPLE ? 4 : 0][row + l] = e;
+                  },
+                  [&] {
+                      if (l < (SAMPLE ? 10 : 3)) {
+#pragma unroll
+                          for (int k = 0; k < COOP_LANES; k += 4) {
+                              const float4 gr = *reinterpret_cast<const float4 *>(pg + k),
+                                           da = *reinterpret_cast<const float4 *>(pa + k);
+                              float4 db = da;
+                              if (SAMPLE) db = *reinterpret_cast<const float4 *>(pb + k);
+                              one(gr.x, da.x, db.x);
+                              one(gr.y, da.y, db.y);
+                              one(gr.z, da.z, db.z);
+                              one(gr.w, da.w, db.w);
+                          }
+                      }
+                  });
+        if (l < (SAMPLE ? 10 : 3)) s_sum[at][l] = acc;
+    }
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    const int lane = threadIdx.x, li = li0 + lane, g = off + min(li, n - 1);
+    const float *r = s_sum[lane];
+    float w[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (SAMPLE) {
+#pragma unroll
+        for (int k = 0; k < 6; k++) w[k] = -0.5f * r[3 + k];
+        w[6] = (POT == RC_POT_SC ? 0.5f * p.eps : 2.0f * p.eps) * r[9];
+    }
+    finish_atom<POT, 32>(p, a, cur, mode, slot, step_index, c, g, li < n, XG[g], s_tab, X + off, r[0], r[1], r[2], w[0], w[1],
+                         w[2], w[3], w[4], w[5], w[6]);
 }
 
 // Eq. PK1 (Sec. 2.2): per cell, the sum over ordered pairs inside rc of
@@ -679,38 +868,62 @@ void rc_prepare_staged(int max_cell_atoms) {
     prepare_density<false>(bytes);
 }
 
-void rc_launch_density(const KParams &p, const KArrays &a, int cur, int n_tiles, int tpa, int stage_atoms,
+// Largest number of tiles for which the cooperative walk is taken: it executes
+// more instructions than one lane per atom and wins while those leave the chip
+// idle.  us per MD step, one lane / cooperative: LJ copper 18 / 14 (28 tiles),
+// 37 / 21 (70), 43 / 33 (140), 49 / 47 (280), 52 / 58 (420); Sutton-Chen 67 / 32
+// (64), 99 / 68 (224), 110 / 95 (320), 140 / 177 (640); Kremer-Grest 32 / 18 (80),
+// 46 / 40 (240), 47 / 46 (320), 52 / 64 (480).
+int rc_coop_max_tiles(int n_sm) { return 2 * n_sm; }
+
+namespace {
+// CTAs per SM it is compiled for: two (64 registers) while they hold the whole
+// batch, else three (40 registers; Kremer-Grest, 240 tiles: 44 -> 40 us)
+bool coop_two(const KParams &p, int coop_tiles) { return coop_tiles * COOP_PER_TILE <= 2 * p.n_sm; }
+}  // namespace
+
+void rc_launch_density(const KParams &p, const KArrays &a, int cur, int n_tiles, int tpa, int stage_atoms, int coop_tiles,
                        cudaStream_t s) {
+    const bool m6 = p.sc_m == 6.0f;
     const int smem = stage_atoms * 16;
-    if (stage_atoms > 0) {
-        if (p.sc_m == 6.0f) launch_density_m<true, true>(p, a, cur, n_tiles, tpa, smem, s);
+    if (coop_tiles > 0) {
+        const auto k = coop_two(p, coop_tiles) ? (m6 ? k_density_coop<true, 2> : k_density_coop<false, 2>)
+                                               : (m6 ? k_density_coop<true, 3> : k_density_coop<false, 3>);
+        rc_launch_pdl(k, coop_tiles * COOP_PER_TILE, COOP_THREADS, 0, s, 1, p, a, cur);
+    } else if (stage_atoms > 0) {
+        if (m6) launch_density_m<true, true>(p, a, cur, n_tiles, tpa, smem, s);
         else launch_density_m<false, true>(p, a, cur, n_tiles, tpa, smem, s);
     } else {
-        if (p.sc_m == 6.0f) launch_density_m<true, false>(p, a, cur, n_tiles, tpa, 0, s);
+        if (m6) launch_density_m<true, false>(p, a, cur, n_tiles, tpa, 0, s);
         else launch_density_m<false, false>(p, a, cur, n_tiles, tpa, 0, s);
     }
 }
 
+namespace {
+
+template <int POT, bool M6>
+void launch_force(const KParams &p, const KArrays &a, int cur, int n_tiles, int tpa, int mode, int slot, int step_index,
+                  int stage_atoms, int coop_tiles, cudaStream_t s) {
+    const bool sample = slot >= 0 || mode == MODE_EVAL;
+    if (coop_tiles > 0) {
+        const auto k = coop_two(p, coop_tiles) ? (sample ? k_force_coop<POT, M6, true, 2> : k_force_coop<POT, M6, false, 2>)
+                                               : (sample ? k_force_coop<POT, M6, true, 3> : k_force_coop<POT, M6, false, 3>);
+        rc_launch_pdl(k, coop_tiles * COOP_PER_TILE, COOP_THREADS, 0, s, 1, p, a, cur, mode, slot, step_index);
+    } else if (stage_atoms > 0)
+        launch_force_pot<POT, M6, true>(p, a, cur, n_tiles, tpa, mode, slot, step_index, stage_atoms * 16, s);
+    else
+        launch_force_pot<POT, M6, false>(p, a, cur, n_tiles, tpa, mode, slot, step_index, 0, s);
+}
+
+}  // namespace
+
 void rc_launch_force(const KParams &p, const KArrays &a, int cur, int n_tiles, int tpa, int mode, int slot,
-                     int step_index, int stage_atoms, cudaStream_t s) {
-    const bool m69 = p.sc_m == 6.0f && p.sc_n == 9.0f;
-    const int smem = stage_atoms * 16;
-    const bool st = stage_atoms > 0;
-    if (p.pot == RC_POT_SC) {
-        if (m69) {
-            if (st) launch_force_pot<RC_POT_SC, true, true>(p, a, cur, n_tiles, tpa, mode, slot, step_index, smem, s);
-            else launch_force_pot<RC_POT_SC, true, false>(p, a, cur, n_tiles, tpa, mode, slot, step_index, 0, s);
-        } else {
-            if (st) launch_force_pot<RC_POT_SC, false, true>(p, a, cur, n_tiles, tpa, mode, slot, step_index, smem, s);
-            else launch_force_pot<RC_POT_SC, false, false>(p, a, cur, n_tiles, tpa, mode, slot, step_index, 0, s);
-        }
-    } else if (p.pot == RC_POT_KG) {
-        if (st) launch_force_pot<RC_POT_KG, false, true>(p, a, cur, n_tiles, tpa, mode, slot, step_index, smem, s);
-        else launch_force_pot<RC_POT_KG, false, false>(p, a, cur, n_tiles, tpa, mode, slot, step_index, 0, s);
-    } else {
-        if (st) launch_force_pot<RC_POT_LJ, false, true>(p, a, cur, n_tiles, tpa, mode, slot, step_index, smem, s);
-        else launch_force_pot<RC_POT_LJ, false, false>(p, a, cur, n_tiles, tpa, mode, slot, step_index, 0, s);
-    }
+                     int step_index, int stage_atoms, int coop_tiles, cudaStream_t s) {
+    const auto go = p.pot == RC_POT_KG   ? launch_force<RC_POT_KG, false>
+                    : p.pot == RC_POT_LJ ? launch_force<RC_POT_LJ, false>
+                    : p.sc_m == 6.0f && p.sc_n == 9.0f ? launch_force<RC_POT_SC, true>
+                                                       : launch_force<RC_POT_SC, false>;
+    go(p, a, cur, n_tiles, tpa, mode, slot, step_index, stage_atoms, coop_tiles, s);
 }
 
 void rc_launch_static_pk1(const KParams &p, const KArrays &a, int cur, int n_tiles, const float *mcell, double *acc,

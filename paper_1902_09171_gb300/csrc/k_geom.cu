@@ -275,6 +275,25 @@ __global__ void __launch_bounds__(RC_TILE) k_keep_frozen(KArrays a, int cur_new)
     (cur_new ? a.x1 : a.x0)[g] = (cur_new ? a.x0 : a.x1)[g];
 }
 
+// Tiles of the active cells in order: block c counts the tiles of the active
+// cells before cell c and writes its own cell's.
+__global__ void __launch_bounds__(RC_TILE) k_active_tiles(KArrays a, int n_cells) {
+    __shared__ int s_part[RC_TILE / 32];
+    const int c = blockIdx.x;
+    const auto tiles = [&](int k) { return a.active[k] ? (a.cell_n[k] + RC_TILE - 1) / RC_TILE : 0; };
+    int before = 0;
+    for (int k = threadIdx.x; k < c; k += RC_TILE) before += tiles(k);
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) before += __shfl_xor_sync(0xffffffffu, before, d);
+    if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = before;
+    __syncthreads();
+    before = 0;
+    for (int w = 0; w < RC_TILE / 32; w++) before += s_part[w];
+    const int own = tiles(c);
+    for (int k = threadIdx.x; k < own; k += RC_TILE) a.act_tiles[before + k] = a.cell_tile0[c] + k;
+    if (c == n_cells - 1 && threadIdx.x == 0) *a.n_act = before + own;
+}
+
 __global__ void k_advance(unsigned long long *evals, const int *active, int n_cells, int n) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c < n_cells && active[c]) evals[c] += (unsigned long long)n;
@@ -305,6 +324,10 @@ void rc_launch_stress(const double *series, int n_avg, int series_cap, const dou
 
 void rc_launch_keep_frozen(const KArrays &a, int cur_new, int n_tiles, cudaStream_t s) {
     k_keep_frozen<<<n_tiles, RC_TILE, 0, s>>>(a, cur_new);
+}
+
+void rc_launch_active_tiles(const KArrays &a, int n_cells, cudaStream_t s) {
+    k_active_tiles<<<n_cells, RC_TILE, 0, s>>>(a, n_cells);
 }
 
 void rc_launch_advance(unsigned long long *evals, const int *active, int n_cells, int n, cudaStream_t s) {

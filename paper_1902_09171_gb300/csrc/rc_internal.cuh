@@ -53,6 +53,7 @@ struct KParams {
     int n_tiles;          // tiles of RC_TILE atoms in the batch
     int n_sm;             // SMs of the device (tile order of the pair kernels)
     int wait_polls;       // polls of a bounded device-side wait before it gives up
+    int masked;           // cells are switched off: the pair kernels take their tiles from act_tiles
 };
 
 struct KArrays {
@@ -67,6 +68,7 @@ struct KArrays {
     int *status;
     int *need_rebuild, *built;
     unsigned long long *rebuilds;  // per cell: neighbour-list builds so far
+    int *act_tiles, *n_act;  // tiles of the active cells, in order, and their number (when masked)
     const int *active;   // per cell: 0 = skipped by every MD kernel (state frozen)
     const unsigned long long *evals;
     double *series;      // [cell][slot][RC_SAMPLE_W]
@@ -242,10 +244,14 @@ void rc_launch_sort(const KParams &p, const KArrays &a, int cur, int n_cells, cu
 void rc_launch_nlist(const KParams &p, const KArrays &a, int cur, int n_cells, cudaStream_t s);
 // stage_atoms > 0: every CTA first copies its whole r-cell (stage_atoms = the
 // largest cell of the batch) into shared memory and gathers neighbours there
+// coop_tiles > 0: the cooperative walk on that many tiles (of the active ones, when masked)
 void rc_launch_density(const KParams &p, const KArrays &a, int cur, int n_tiles, int tpa, int stage_atoms,
-                       cudaStream_t s);
+                       int coop_tiles, cudaStream_t s);
 void rc_launch_force(const KParams &p, const KArrays &a, int cur, int n_tiles, int tpa, int mode, int slot,
-                     int step_index, int stage_atoms, cudaStream_t s);
+                     int step_index, int stage_atoms, int coop_tiles, cudaStream_t s);
+int rc_coop_max_tiles(int n_sm);
+// act_tiles and n_act from the activity mask
+void rc_launch_active_tiles(const KArrays &a, int n_cells, cudaStream_t s);
 int rc_stage_max_atoms();
 void rc_prepare_staged(int max_cell_atoms);
 void rc_launch_deform_impl(const double *F, double *H, double *Rprev, double *Q, double *R, double *Fst, double *dR,

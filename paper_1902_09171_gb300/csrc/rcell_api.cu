@@ -47,6 +47,7 @@ struct rcell_ctx {
     int series_cap = 0;
     int last_n_avg = -1;
     int cur = 0;
+    int n_act = 0;  // tiles of the active cells, -1: a device mask's, not known here
     int tpa = 1;
     int use_graphs = 1;
     int max_cell = 0;    // largest cell of the batch (atoms)
@@ -57,11 +58,11 @@ struct rcell_ctx {
     FireState fire{};
     int *d_fire_left = nullptr;
     cudaGraphExec_t fire_graph = nullptr;  // one captured batch of FIRE iterations
-    double fire_key[5] = {0, 0, 0, 0, 0};   // f_tol, dt_max, dmax, tpa, cur it was captured with
+    double fire_key[6] = {0, 0, 0, 0, 0, 0};   // f_tol, dt_max, dmax, tpa, cur, plan it was captured with
     float *d_mcell = nullptr;
     double *d_pk_acc = nullptr;
-    std::map<std::tuple<int, int, int, int>, cudaGraphExec_t> graphs;
-    std::map<std::tuple<int, int, int, int>, long> graph_launches;
+    std::map<std::tuple<int, int, int, int, int>, cudaGraphExec_t> graphs;
+    std::map<std::tuple<int, int, int, int, int>, long> graph_launches;
     std::string err = "ok";
 };
 
@@ -140,6 +141,31 @@ int stage_atoms(const rcell_ctx *c) {
     return (c->staged && c->max_cell <= rc_stage_max_atoms()) ? c->max_cell : 0;
 }
 
+// Tiles the cooperative walk is launched on, 0 where the other one is taken: the
+// whole batch or, when a mask's cells are known, a power of two that holds their
+// tiles (few different graphs; the surplus blocks return at once).
+int coop_tiles(const rcell_ctx *c) {
+    if (c->tpa > 1 || stage_atoms(c) > 0 || c->n_act < 0 || c->n_act > rc_coop_max_tiles(c->kp.n_sm)) return 0;
+    if (!c->kp.masked) return c->n_tiles;
+    int t = 1;
+    while (t < c->n_act) t *= 2;
+    return t;
+}
+
+// the activity mask in force, on(cell), where the host knows it
+template <class On>
+void know_mask(rcell_ctx *c, On &&on) {
+    c->n_act = 0;
+    c->kp.masked = 0;
+    for (int k = 0; k < c->n_cells; k++) {
+        if (on(k)) c->n_act += c->h_ntiles[k];
+        else c->kp.masked = 1;
+    }
+}
+
+// what a captured graph depends on beyond its steps and buffers
+int plan(const rcell_ctx *c) { return 2 * coop_tiles(c) + c->kp.masked; }
+
 // enqueue the neighbour rebuild (when scheduled) and the force launches of one
 // step; returns the number of kernels enqueued
 long enqueue_step(rcell_ctx *c, int mode, int slot, int step_index) {
@@ -148,10 +174,10 @@ long enqueue_step(rcell_ctx *c, int mode, int slot, int step_index) {
     rc_launch_nlist(c->kp, c->ka, c->cur, c->n_cells, c->stream);
     k += 2;
     if (c->kp.pot == RC_POT_SC) {
-        rc_launch_density(c->kp, c->ka, c->cur, c->n_tiles, c->tpa, stage_atoms(c), c->stream);
+        rc_launch_density(c->kp, c->ka, c->cur, c->n_tiles, c->tpa, stage_atoms(c), coop_tiles(c), c->stream);
         k++;
     }
-    rc_launch_force(c->kp, c->ka, c->cur, c->n_tiles, c->tpa, mode, slot, step_index, stage_atoms(c), c->stream);
+    rc_launch_force(c->kp, c->ka, c->cur, c->n_tiles, c->tpa, mode, slot, step_index, stage_atoms(c), coop_tiles(c), c->stream);
     k++;
     return k;
 }
@@ -326,6 +352,9 @@ int rcell_create(const rcell_params *params, int n_cells, const rcell_init *cell
         CKC(c, cudaMemcpy(d_active, ones.data(), sizeof(int) * n_cells, cudaMemcpyHostToDevice));
     }
     A.active = d_active;
+    CKC(c, dalloc(L, &A.act_tiles, tiles));
+    CKC(c, dalloc(L, &A.n_act, 1));
+    c->n_act = c->n_tiles;
     CKC(c, dalloc(L, &c->d_evals, n_cells));
     CKC(c, dalloc(L, &A.eval_acc, 8 * (size_t)n_cells));
     CKC(c, dalloc(L, &c->d_H, 9 * (size_t)n_cells));
@@ -456,7 +485,7 @@ int rcell_run(rcell_ctx *c, int n_steps, int n_avg) {
     int e = ensure_series(c, n_avg);
     if (e != RC_OK) return e;
     if (c->use_graphs) {
-        auto key = std::make_tuple(n_steps, n_avg, c->cur, c->tpa);
+        auto key = std::make_tuple(n_steps, n_avg, c->cur, c->tpa, plan(c));
         auto it = c->graphs.find(key);
         if (it == c->graphs.end()) {
             cudaGraph_t g = nullptr;
@@ -488,7 +517,15 @@ int rcell_set_active(rcell_ctx *c, const int *mask, int where) {
     if (!c || !mask) return RC_EINVAL;
     CKC(c, cudaMemcpyAsync((void *)c->ka.active, mask, sizeof(int) * c->n_cells,
                            where == RC_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, c->stream));
-    if (where == RC_HOST) CKC(c, cudaStreamSynchronize(c->stream));
+    rc_launch_active_tiles(c->ka, c->n_cells, c->stream);
+    CKC(c, cudaGetLastError());
+    if (where == RC_HOST) {
+        know_mask(c, [&](int k) { return mask[k] != 0; });
+        CKC(c, cudaStreamSynchronize(c->stream));
+    } else {
+        c->kp.masked = 1;
+        c->n_act = -1;
+    }
     return RC_OK;
 }
 
@@ -714,8 +751,8 @@ int rcell_minimize(rcell_ctx *c, int max_iter, double f_tol, double dt0, double 
                                      (float)dmax, k == nb - 1 ? c->d_fire_left : nullptr, c->stream);
         }
     };
-    const double key[5] = {f_tol, dt_max, dmax, (double)c->tpa, (double)c->cur};
-    if (c->use_graphs && (!c->fire_graph || !std::equal(key, key + 5, c->fire_key))) {
+    const double key[6] = {f_tol, dt_max, dmax, (double)c->tpa, (double)c->cur, (double)plan(c)};
+    if (c->use_graphs && (!c->fire_graph || !std::equal(key, key + 6, c->fire_key))) {
         if (c->fire_graph) cudaGraphExecDestroy(c->fire_graph);
         c->fire_graph = nullptr;
         cudaGraph_t g = nullptr;
@@ -725,7 +762,7 @@ int rcell_minimize(rcell_ctx *c, int max_iter, double f_tol, double dt0, double 
         cudaError_t ce = cudaGraphInstantiate(&c->fire_graph, g, 0);
         cudaGraphDestroy(g);
         if (ce != cudaSuccess) { c->fire_graph = nullptr; return fail(c, RC_ECUDA, "FIRE graph instantiation"); }
-        std::copy(key, key + 5, c->fire_key);
+        std::copy(key, key + 6, c->fire_key);
     }
     for (int it0 = 0; it0 < max_iter; it0 += batch) {
         const int nb = std::min(batch, max_iter - it0);
@@ -757,7 +794,7 @@ int rcell_stress_static(rcell_ctx *c, double *sigma, double *P, int where) {
     rc_launch_static_prep(c->d_H, c->d_H0, c->d_mcell, c->d_pk_acc, nc, c->stream);
     rc_launch_sort(c->kp, c->ka, c->cur, nc, c->stream);
     rc_launch_nlist(c->kp, c->ka, c->cur, c->n_cells, c->stream);
-    if (c->kp.pot == RC_POT_SC) rc_launch_density(c->kp, c->ka, c->cur, c->n_tiles, 1, 0, c->stream);
+    if (c->kp.pot == RC_POT_SC) rc_launch_density(c->kp, c->ka, c->cur, c->n_tiles, 1, 0, 0, c->stream);
     rc_launch_static_pk1(c->kp, c->ka, c->cur, c->n_tiles, c->d_mcell, c->d_pk_acc, c->stream);
     rc_launch_static_finish(c->d_pk_acc, c->d_H0, c->d_Q, c->d_F, pconv_of(c->prm.units), c->d_P, c->d_sig_fem,
                             c->ka.status, nc, c->stream);
@@ -891,9 +928,10 @@ int rcell_profile_kernels(rcell_ctx *c, int n_steps, double *ms_out) {
         CKC(c, cudaEventRecord(ev[1], c->stream));
         rc_launch_nlist(c->kp, c->ka, c->cur, c->n_cells, c->stream);
         CKC(c, cudaEventRecord(ev[2], c->stream));
-        if (c->kp.pot == RC_POT_SC) rc_launch_density(c->kp, c->ka, c->cur, c->n_tiles, c->tpa, stage_atoms(c), c->stream);
+        if (c->kp.pot == RC_POT_SC) rc_launch_density(c->kp, c->ka, c->cur, c->n_tiles, c->tpa, stage_atoms(c), coop_tiles(c), c->stream);
         CKC(c, cudaEventRecord(ev[3], c->stream));
-        rc_launch_force(c->kp, c->ka, c->cur, c->n_tiles, c->tpa, mode, slot, s, stage_atoms(c), c->stream);
+        rc_launch_force(c->kp, c->ka, c->cur, c->n_tiles, c->tpa, mode, slot, s, stage_atoms(c), coop_tiles(c),
+                        c->stream);
         CKC(c, cudaEventRecord(ev[4], c->stream));
         CKC(c, cudaEventSynchronize(ev[4]));
         lap(0, 1, 0);
@@ -1140,6 +1178,7 @@ int fe_step_surrogate(fe_ctx *fe, rcell_ctx *rc, sur_ctx *sur, double lambda, in
     for (int j = 0; j < max_k; j++) {
         fe_launch_replay_mask(md_flag, fe->d_nfrozen, j, fe->d_rmask, ne, st);
         if ((e = rcell_set_active(rc, fe->d_rmask, RC_DEVICE)) != RC_OK) return e;
+        know_mask(rc, [&](int k) { return fe->h_flag[k] != 0 && fe->h_nfrozen[k] > j; });
         if ((e = rcell_set_deformation(rc, fe->d_Fhist + (size_t)j * ne * 9, RC_DEVICE)) != RC_OK) return e;
         if ((e = rcell_run(rc, n_steps, n_avg)) != RC_OK) return e;  // the all-MD kernel sequence
     }
@@ -1147,6 +1186,7 @@ int fe_step_surrogate(fe_ctx *fe, rcell_ctx *rc, sur_ctx *sur, double lambda, in
     //    r-cell state)
     if (nmd > 0) {
         if ((e = rcell_set_active(rc, md_flag, RC_DEVICE)) != RC_OK) return e;
+        know_mask(rc, [&](int k) { return fe->h_flag[k] != 0; });
         if ((e = rcell_set_deformation(rc, fe->d_F, RC_DEVICE)) != RC_OK) return e;
         if ((e = rcell_run(rc, n_steps, n_avg)) != RC_OK) return e;
         if ((e = rcell_stress(rc, nullptr, nullptr, fe->d_Pmd, RC_DEVICE)) != RC_OK) return e;
