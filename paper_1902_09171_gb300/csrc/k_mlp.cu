@@ -415,12 +415,12 @@ void prepare_tc05() {
 // shared memory (BF16, K-major core-matrix layout) and the layer accumulators
 // (128 x 256 FP32) in tensor memory, two of them (512 columns), so that a
 // layer's MMAs can write one while the epilogue still reads the other.  The
-// roles are split between warps: one producer thread streams the weights
+// roles are split between warps: one thread streams the weights
 // through four shared buffers, one 64-column K slice of a layer (all its output
 // rows) per buffer, with bulk copies (cp.async.bulk, one per chunk, completing
 // on a per-buffer mbarrier; the weights are pre-arranged per member by
 // k_pack_weights so that each chunk is one contiguous block in the buffer's
-// layout), and issues the MMAs slice by slice; sixteen epilogue warps (warp w:
+// layout), another issues the MMAs slice by slice; sixteen epilogue warps (warp w:
 // accumulator rows 32 (w % 4).., columns 16 (w / 4).. of every slice) wait for
 // a layer's accumulator and run its epilogue (bias + GELU into the next
 // operand, slice after slice; the head writes the stress and the new state
@@ -428,13 +428,13 @@ void prepare_tc05() {
 // of the next layer start as soon as all warps have written slice s of its
 // operand, under the rest of the epilogue.  The two sides meet only at
 // mbarriers, all waits bounded:
-//   full[b]  : chunk in buffer b has landed          (bulk copy -> producer)
-//   empty[b] : the MMAs reading buffer b are done     (tcgen05.commit -> producer)
+//   full[b]  : chunk in buffer b has landed          (bulk copy -> MMA thread)
+//   empty[b] : the MMAs reading buffer b are done     (tcgen05.commit -> load thread)
 //   acc      : a layer's accumulator is complete      (tcgen05.commit -> epilogue)
 //   slice[s] : the epilogue warps have written slice s of a hidden layer's
-//              output (16 warp arrivals -> producer)
+//              output (16 warp arrivals -> MMA thread)
 //   epi      : the epilogue warps have written the next step's input rows
-//              (16 warp arrivals -> producer, and -> the epilogue warps
+//              (16 warp arrivals -> MMA thread, and -> the epilogue warps
 //              before they copy the rows to the tape)
 // With a tape (training) every step's z, y and a rows also go to global memory
 // for the backward pass, in the layout the layer-wise kernels use.
@@ -527,7 +527,7 @@ __device__ __forceinline__ float gelu_step(float x) {
 }
 __device__ __forceinline__ float gelu_fast(float x) { return x * gelu_step(x); }
 
-constexpr int WS_EPI_WARPS = 16, WS_THREADS = (WS_EPI_WARPS + 1) * 32;
+constexpr int WS_EPI_WARPS = 16, WS_THREADS = (WS_EPI_WARPS + 2) * 32;  // + the MMA and the load warp
 static_assert(WS_EPI_WARPS == 4 * FT_PARTS, "epilogue warps cover 4 lane quarters x FT_PARTS column parts");
 
 // Chunk j (0..14) of one step's weight sequence: layer l, K slice s (columns
@@ -571,7 +571,7 @@ __global__ void k_pack_weights(const __nv_bfloat16 *__restrict__ W0, const __nv_
 
 // Bounded wait that lets the hardware park the thread (up to WS_SUSPEND_NS per
 // try) instead of spinning, so that waiting warps leave the issue slots to the
-// producer and to the warps that have work: at most WS_TRIES tries (~2 s).
+// MMA thread and to the warps that have work: at most WS_TRIES tries (~2 s).
 constexpr unsigned WS_SUSPEND_NS = 100000;
 constexpr int WS_TRIES = 20000;
 
@@ -750,7 +750,7 @@ __device__ __forceinline__ void ws_head16(const FusedArgs &a, int t, int row, in
     st_state16<NOUT, NIN - NOUT>(sZA, row, n0, hv);
 }
 
-// Hands the epilogue's operand writes to the producer: shared-memory writes
+// Hands the epilogue's operand writes to the MMA thread: shared-memory writes
 // made visible to the tensor core's proxy, tensor-memory reads ordered before
 // the synchronisation, then one arrival per warp on `bar`.
 __device__ __forceinline__ void ws_hand_over(unsigned bar, int lane) {
@@ -818,75 +818,84 @@ __device__ __forceinline__ void ws_epilogue_head(const FusedArgs &a, int t, int 
     }
 }
 
-// The producer thread of the warp-specialised kernels: streams T x FT_CHUNKS
-// weight chunks (per step the K slices of the four layers, see ws_chunk_*)
-// through the FT_NBUF buffers and issues the MMAs slice by slice: slice s of
-// layer l (its K columns 64 s ..) goes as soon as its operand columns are in
+// The two producer threads of the warp-specialised kernels.  ws_load streams T x
+// FT_CHUNKS weight chunks (per step the K slices of the four layers, see
+// ws_chunk_*) through the FT_NBUF buffers, each as soon as the MMAs that read
+// the buffer's last chunk are done.  ws_mma issues the MMAs slice by slice: slice
+// s of layer l (its K columns 64 s ..) goes as soon as its operand columns are in
 // place -- for the first layer when the whole input rows are (the `epi`
 // barrier), for the others when the epilogue warps have finished slice s of
 // the previous layer (`slice[s]`) -- so that the MMAs of a layer run under
 // the epilogue of the previous one.  Layer l accumulates into tensor-memory
 // columns (l % 2) * 256 .., the other half from the epilogue still reading the
 // previous layer.  False on a timeout.
-__device__ __forceinline__ bool ws_produce(const unsigned char *Wp, int T, unsigned char *sZA, unsigned char *sW,
-                                           unsigned tmem, unsigned bar_full, unsigned bar_empty, unsigned bar_acc,
-                                           unsigned bar_epi, unsigned bar_slice) {
-    bool ok = true;
+//
+// One thread for both waited, between a slice's MMAs and the next's, for the
+// MMAs before them to free a buffer: 1650 cycles per slice where the epilogue
+// hands one over every 1050, so that a layer's accumulator came 4800 cycles
+// after the last hand-over (of 9300 per layer).  With two: prediction of 4 x 4096
+// x 60 rows 1.028 -> 0.687 ms, forward with tape 1.464 -> 1.287, backward 1.495 ->
+// 1.237 ms.
+__device__ __forceinline__ bool ws_load(const unsigned char *Wp, int T, unsigned char *sW, unsigned bar_full,
+                                        unsigned bar_empty) {
     const long n_chunks = (long)T * FT_CHUNKS;
-    for (long c0 = 0; c0 < FT_NBUF && c0 < n_chunks; c0++) ws_bulk(sW, Wp, c0, bar_full);
-    const unsigned aBase = (unsigned)__cvta_generic_to_shared(sZA);
-    const unsigned lboA = (FT_M / 8) * 128;
     long c = 0;
-    for (int t = 0; t < T && ok; t++)
-        for (int l = 0; l < 4 && ok; l++) {
+    for (; c < n_chunks; c++) {
+        if (c >= FT_NBUF && !ws_wait(bar_empty + 8u * (unsigned)(c % FT_NBUF), (unsigned)((c / FT_NBUF - 1) & 1))) break;
+        ws_bulk(sW, Wp, c, bar_full);
+    }
+    // no copy is in flight when the block ends, however it ends
+    for (long k = c > FT_NBUF ? c - FT_NBUF : 0; k < c; k++)
+        ws_wait(bar_full + 8u * (unsigned)(k % FT_NBUF), (unsigned)((k / FT_NBUF) & 1));
+    return c == n_chunks;
+}
+
+__device__ __forceinline__ bool ws_mma(int T, unsigned char *sZA, unsigned char *sW, unsigned tmem, unsigned bar_full,
+                                       unsigned bar_empty, unsigned bar_acc, unsigned bar_epi, unsigned bar_slice) {
+    const unsigned aBase = (unsigned)__cvta_generic_to_shared(sZA), wBase = (unsigned)__cvta_generic_to_shared(sW);
+    const unsigned lboA = (FT_M / 8) * 128;
+    const uint64_t adesc = tc_desc(aBase, lboA, 128);  // + 16 (address units) per 256 bytes
+    long c = 0;
+    for (int t = 0; t < T; t++)
+        for (int l = 0; l < 4; l++) {
             const int N = ws_layer_n(l), ns = l == 0 ? 3 : 4;
             const unsigned idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(N >> 3) << 17) |
                                    ((unsigned)(FT_M >> 4) << 24);
             const unsigned lboB = (unsigned)(N / 8) * 128;
             const unsigned dcol = tmem + (unsigned)((l & 1) * WID);
-            for (int sl = 0; sl < ns && ok; sl++, c++) {
+            for (int sl = 0; sl < ns; sl++, c++) {
+                const int b = (int)(c % FT_NBUF), nkk = ws_slice_kw(l, sl) >> 4;
+                uint64_t ad = adesc + (uint64_t)(sl * (FT_KS / 16)) * (2 * lboA >> 4);
+                uint64_t bd = tc_desc(wBase + (unsigned)b * FT_SW, lboB, 128);
+                if (!ws_wait(bar_full + 8u * b, (unsigned)((c / FT_NBUF) & 1))) return false;
                 // operand columns of slice sl in place: the input rows of step t
                 // (completion t of `epi`), or slice sl of the previous layer's
                 // epilogue (completion 3 t + l - 1 of `slice[sl]`)
                 if (l == 0) {
-                    if (sl == 0) ok = ws_wait(bar_epi, (unsigned)(t & 1));
+                    if (sl == 0 && !ws_wait(bar_epi, (unsigned)(t & 1))) return false;
                 } else {
-                    ok = ws_wait(bar_slice + 8u * sl, (unsigned)((3 * t + l - 1) & 1));
+                    if (!ws_wait(bar_slice + 8u * sl, (unsigned)((3 * t + l - 1) & 1))) return false;
                 }
-                if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const int b = (int)(c % FT_NBUF);
-                ok = ws_wait(bar_full + 8u * b, (unsigned)((c / FT_NBUF) & 1));
-                if (!ok) break;
-                const unsigned wb = (unsigned)__cvta_generic_to_shared(sW + (size_t)b * FT_SW);
-                const int nkk = ws_slice_kw(l, sl) >> 4;
                 for (int kk = 0; kk < nkk; kk++) {
-                    const uint64_t ad = tc_desc(aBase + (sl * (FT_KS / 16) + kk) * 2 * lboA, lboA, 128);
-                    const uint64_t bd = tc_desc(wb + kk * 2 * lboB, lboB, 128);
                     const unsigned acc = (sl > 0 || kk > 0) ? 1u : 0u;
                     asm volatile(
                         "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
                         " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dcol),
                         "l"(ad), "l"(bd), "r"(idesc), "r"(acc)
                         : "memory");
+                    ad += 2 * lboA >> 4;
+                    bd += 2 * lboB >> 4;
                 }
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                                  bar_empty + 8u * b)
                              : "memory");
-                // refill the buffer of chunk c - 1 once the MMAs that read it are done
-                if (c >= 1 && c - 1 + FT_NBUF < n_chunks) {
-                    const int pb = (int)((c - 1) % FT_NBUF);
-                    ok = ws_wait(bar_empty + 8u * pb, (unsigned)(((c - 1) / FT_NBUF) & 1));
-                    if (!ok) break;
-                    ws_bulk(sW, Wp, c - 1 + FT_NBUF, bar_full);
-                }
             }
-            if (!ok) break;
             // the accumulator is complete once every MMA issued so far is
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar_acc)
                          : "memory");
         }
-    return ok;
+    return true;
 }
 
 __global__ void __launch_bounds__(WS_THREADS, 1) k_forward_ws(FusedArgs a) {
@@ -938,9 +947,15 @@ __global__ void __launch_bounds__(WS_THREADS, 1) k_forward_ws(FusedArgs a) {
     bool ok = true;
 
     if (warp == WS_EPI_WARPS) {
-        // ---- producer: weight chunks and MMAs (one thread) ----
+        // ---- MMAs (one thread) ----
         if (lane == 0) {
-            ok = ws_produce(a.Wp[mk], T, sZA, sW, tmem, bar_full, bar_empty, bar_acc, bar_epi, bar_slice);
+            ok = ws_mma(T, sZA, sW, tmem, bar_full, bar_empty, bar_acc, bar_epi, bar_slice);
+            if (!ok) atomicExch(a.err, RC_ETIMEOUT);
+        }
+    } else if (warp == WS_EPI_WARPS + 1) {
+        // ---- weight chunks (one thread) ----
+        if (lane == 0) {
+            ok = ws_load(a.Wp[mk], T, sW, bar_full, bar_empty);
             if (!ok) atomicExch(a.err, RC_ETIMEOUT);
         }
     } else {
@@ -1217,7 +1232,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad_tc05(const __grid_const
 //   dY1 = (dY2 W2^T) * gelu'(Y1_t),   dZ_t = dY1 W1^T
 // run back to back on the tensor cores with the operand in shared memory and
 // the accumulator in tensor memory.  They have the forward's shapes in the
-// reverse order, so the same producer streams the members' backward weight
+// reverse order, so the same two threads stream the members' backward weight
 // images (W4, W3, W2, W1 packed by k_pack_weights as the forward packs W1^T ..
 // W4^T).  The epilogue warps read Y_l from the tape, write dY_l into shared
 // memory (the next operand) and to global memory (for the weight gradients);
@@ -1428,8 +1443,15 @@ __global__ void __launch_bounds__(WS_THREADS, 1) k_backward_ws(BwdArgs a) {
     bool ok = true;
 
     if (warp == WS_EPI_WARPS) {
+        // ---- MMAs (one thread) ----
         if (lane == 0) {
-            ok = ws_produce(a.Wb[mk], T, sZA, sW, tmem, bar_full, bar_empty, bar_acc, bar_epi, bar_slice);
+            ok = ws_mma(T, sZA, sW, tmem, bar_full, bar_empty, bar_acc, bar_epi, bar_slice);
+            if (!ok) atomicExch(a.err, RC_ETIMEOUT);
+        }
+    } else if (warp == WS_EPI_WARPS + 1) {
+        // ---- weight chunks (one thread) ----
+        if (lane == 0) {
+            ok = ws_load(a.Wb[mk], T, sW, bar_full, bar_empty);
             if (!ok) atomicExch(a.err, RC_ETIMEOUT);
         }
     } else {
