@@ -63,12 +63,33 @@ __global__ void k_geometry(const double *__restrict__ X, const int *__restrict__
 
 // prescribed DOFs take lambda val; with an affine predictor g of the load
 // increment, every free DOF first moves by (lambda - lambda_prev) g
+__device__ __forceinline__ double bc_value(const int *__restrict__ mask, const double *__restrict__ val,
+                                           const double *__restrict__ g, double lambda, double dlambda, const double *d,
+                                           int q) {
+    // (explicit rounding: every kernel that asks has the same bits)
+    if (mask[q]) return __dmul_rn(lambda, val[q]);
+    return g ? __fma_rn(dlambda, g[q], d[q]) : d[q];
+}
+
 __global__ void k_apply_bc(const int *__restrict__ mask, const double *__restrict__ val,
                            const double *__restrict__ g, double lambda, double dlambda, double *d, int n3) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n3) return;
-    if (mask[q]) d[q] = lambda * val[q];
-    else if (g) d[q] += dlambda * g[q];
+    if (q < n3) d[q] = bc_value(mask, val, g, lambda, dlambda, d, q);
+}
+
+// F_e = I + sum_a d_a (x) grad N_a, disp(q) = displacement of DOF q
+template <int NPE, class Disp>
+__device__ __forceinline__ void element_F(const int *__restrict__ conn, const double *__restrict__ gradN, int e, Disp &&disp,
+                                          double (&G)[9]) {
+    for (int k = 0; k < 9; k++) G[k] = k % 4 == 0 ? 1.0 : 0.0;
+    for (int a = 0; a < NPE; a++) {
+        const int q = 3 * conn[NPE * e + a];
+        const double *ga = gradN + 3 * NPE * e + 3 * a;
+        for (int i = 0; i < 3; i++) {
+            const double di = disp(q + i);
+            for (int J = 0; J < 3; J++) G[3 * i + J] = __fma_rn(di, ga[J], G[3 * i + J]);
+        }
+    }
 }
 
 template <int NPE>
@@ -76,13 +97,8 @@ __global__ void k_F(const int *__restrict__ conn, const double *__restrict__ gra
                     double *F, int ne) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= ne) return;
-    double G[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1};
-    for (int a = 0; a < NPE; a++) {
-        const double *da = d + 3 * conn[NPE * e + a];
-        const double *ga = gradN + 3 * NPE * e + 3 * a;
-        for (int i = 0; i < 3; i++)
-            for (int J = 0; J < 3; J++) G[3 * i + J] += da[i] * ga[J];
-    }
+    double G[9];
+    element_F<NPE>(conn, gradN, e, [&](int q) { return d[q]; }, G);
     for (int k = 0; k < 9; k++) F[9 * e + k] = G[k];
 }
 
@@ -90,12 +106,10 @@ __global__ void k_F(const int *__restrict__ conn, const double *__restrict__ gra
 // gamma_{alpha a} = (h_{alpha a} - (sum_b h_{alpha b} X_b) . grad N_a) / 8,
 // h = (eta zeta, zeta xi, xi eta, xi eta zeta) at the nodes, q_alpha = sum_b gamma_{alpha b} d_b.
 template <int NPE>
-__global__ void k_fint(const double *__restrict__ X, const int *__restrict__ conn, const double *__restrict__ gradN,
-                       const double *__restrict__ V0, const double *__restrict__ P, const double *__restrict__ d,
-                       double hg, double *fint, int ne) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= ne) return;
-    const double *g = gradN + 3 * NPE * e, *Pe = P + 9 * e;
+__device__ __forceinline__ void element_fint(const double *__restrict__ X, const int *__restrict__ conn,
+                                             const double *__restrict__ gradN, const double *__restrict__ V0,
+                                             const double *Pe, const double *__restrict__ d, double hg, double *fint, int e) {
+    const double *g = gradN + 3 * NPE * e;
     const double V = V0[e];
     double fe[3 * NPE];
     for (int a = 0; a < NPE; a++)
@@ -129,6 +143,14 @@ __global__ void k_fint(const double *__restrict__ X, const int *__restrict__ con
         for (int i = 0; i < 3; i++) atomicAdd(&fint[3 * conn[NPE * e + a] + i], fe[3 * a + i]);
 }
 
+template <int NPE>
+__global__ void k_fint(const double *__restrict__ X, const int *__restrict__ conn, const double *__restrict__ gradN,
+                       const double *__restrict__ V0, const double *__restrict__ P, const double *__restrict__ d,
+                       double hg, double *fint, int ne) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < ne) element_fint<NPE>(X, conn, gradN, V0, P + 9 * e, d, hg, fint, e);
+}
+
 __global__ void k_update(const int *__restrict__ mask, const double *__restrict__ mass, const double *__restrict__ fint,
                          double dt, double damping, double *d, double *v, int n3) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -144,21 +166,6 @@ __global__ void k_update(const int *__restrict__ mask, const double *__restrict_
     d[q] += dt * vn;
 }
 
-// MD-fallback decision per quadrature point with hysteresis: a point trips to MD
-// when the ensemble spread exceeds `on` and, once tripped, stays on MD while the
-// spread exceeds `off`.  Flags: 0 surrogate, 1 tripped (MD), 2 forced MD
-// (start-up increments; a forced point is not tripped).
-__global__ void k_decide(const float *__restrict__ spread, float on, float off, int force_md, int *md_flag, int *n_md,
-                         int ne) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= ne) return;
-    const float sp = spread[e];
-    const int tripped = !(sp <= on) || (md_flag[e] == 1 && !(sp <= off));
-    const int flag = tripped ? 1 : (force_md ? 2 : 0);
-    md_flag[e] = flag;
-    if (flag) atomicAdd(n_md, 1);
-}
-
 // Replay of missed increments: mask of the points that run MD at this increment
 // and still have a recorded deformation at replay position j.
 __global__ void k_replay_mask(const int *__restrict__ md_flag, const int *__restrict__ n_frozen, int j, int *mask,
@@ -168,34 +175,53 @@ __global__ void k_replay_mask(const int *__restrict__ md_flag, const int *__rest
     mask[e] = (md_flag[e] != 0 && n_frozen[e] > j) ? 1 : 0;
 }
 
-// After the step: a point on MD has no missed increment left; a point on the
-// surrogate records this increment's F at the next free position of its history
-// (when all kmax positions are taken, the last one is overwritten, so the
-// history keeps the first kmax - 1 missed increments and the latest).
-__global__ void k_track_frozen(const int *__restrict__ md_flag, const double *__restrict__ F, double *F_hist,
-                               int *n_frozen, int ne, int kmax) {
+// ---------------------------------------------------------------------------
+// The FE step with the surrogate (fe_step_surrogate), three kernels around the
+// members' forward pass.  Every one of them is a few microseconds of launch and
+// latency whatever the mesh, so what one thread per element or DOF can do in
+// sequence is in one kernel, and the flags reach the host in pinned memory that
+// the kernel writes itself.  Against fifteen launches, copies and a memset: 165 ->
+// 113 us per step of 32 points, none on MD.
+// ---------------------------------------------------------------------------
+
+// Per element: F from the displacements that this step's boundary conditions
+// give (k_step_decide stores them), and the surrogate's input.
+template <int NPE>
+__global__ void k_step_begin(FeStepArgs a) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= ne) return;
-    if (md_flag[e] != 0) {
-        n_frozen[e] = 0;
-        return;
-    }
-    const int n = n_frozen[e];
-    const int slot = n < kmax ? n : kmax - 1;
-    for (int k = 0; k < 9; k++) F_hist[((size_t)slot * ne + e) * 9 + k] = F[9 * e + k];
-    n_frozen[e] = n < kmax ? n + 1 : kmax;
+    if (e >= a.ne) return;
+    double G[9];
+    element_F<NPE>(a.conn, a.gradN, e, [&](int q) { return bc_value(a.mask, a.val, a.g, a.lambda, a.dlambda, a.d, q); }, G);
+    for (int k = 0; k < 9; k++) a.F[9 * e + k] = G[k];
+    rc_features(a.F_prev + 9 * e, G, a.u + (size_t)e * 15);
 }
 
-// P = J sigma F^{-T} from the surrogate stress (FE frame) where the point is not on MD
-__global__ void k_merge_P(const int *__restrict__ md_flag, const float *__restrict__ s_sur, const double *__restrict__ F,
-                          const double *__restrict__ P_md, double *P, int ne) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= ne) return;
-    if (md_flag[e]) {
-        for (int k = 0; k < 9; k++) P[9 * e + k] = P_md[9 * e + k];
-        return;
+// Per point: ensemble mean and spread, and the MD-fallback decision with
+// hysteresis: a point trips to MD when the spread exceeds `on` and, once tripped,
+// stays on MD while it exceeds `off`.  Flags: 0 surrogate, 1 tripped (MD), 2
+// forced MD (start-up increments; a forced point is not tripped).  Per DOF: the
+// displacement under the boundary conditions, and a zeroed internal force.
+__global__ void k_step_decide(FeStepArgs a) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < a.n3) {
+        a.d[i] = bc_value(a.mask, a.val, a.g, a.lambda, a.dlambda, a.d, i);
+        a.fint[i] = 0.0;
     }
-    const double *Fe = F + 9 * e;
+    if (i >= a.ne) return;
+    float mu[6];
+    const float sp = rc_ensemble(a.Sm, a.n_members, a.ne, i, a.s_floor, mu);
+    for (int c = 0; c < 6; c++) a.s_mean[(size_t)i * 6 + c] = mu[c];
+    a.spread[i] = sp;
+    if (a.spread_out) a.spread_out[i] = sp;
+    const int tripped = !(sp <= a.on) || (a.md_flag[i] == 1 && !(sp <= a.off));
+    const int flag = tripped ? 1 : (a.force_md ? 2 : 0);
+    a.md_flag[i] = flag;
+    a.host_flag[i] = flag;
+    a.host_frozen[i] = a.n_frozen[i];
+}
+
+// P = J sigma F^{-T} from the surrogate stress (FE frame)
+__device__ __forceinline__ void surrogate_P(const float *sv, const double *Fe, double (&P)[9]) {
     const double J = Fe[0] * (Fe[4] * Fe[8] - Fe[5] * Fe[7]) - Fe[1] * (Fe[3] * Fe[8] - Fe[5] * Fe[6]) +
                      Fe[2] * (Fe[3] * Fe[7] - Fe[4] * Fe[6]);
     double Fi[9];
@@ -208,42 +234,60 @@ __global__ void k_merge_P(const int *__restrict__ md_flag, const float *__restri
     Fi[6] = (Fe[3] * Fe[7] - Fe[4] * Fe[6]) / J;
     Fi[7] = (Fe[1] * Fe[6] - Fe[0] * Fe[7]) / J;
     Fi[8] = (Fe[0] * Fe[4] - Fe[1] * Fe[3]) / J;
-    const float *sv = s_sur + 6 * e;
     const double S[9] = {sv[0], sv[3], sv[4], sv[3], sv[1], sv[5], sv[4], sv[5], sv[2]};
     for (int i = 0; i < 3; i++)
         for (int j = 0; j < 3; j++) {
             double acc = 0.0;
             for (int l = 0; l < 3; l++) acc += S[3 * i + l] * Fi[3 * j + l];
-            P[9 * e + 3 * i + j] = J * acc;
+            P[3 * i + j] = J * acc;
         }
 }
 
-__global__ void k_copy_F(const double *__restrict__ F, double *F_prev, int n) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) F_prev[i] = F[i];
+// Per element: P of the MD where the point is flagged, of the surrogate
+// elsewhere; the internal force; and the point's record of missed increments: a
+// point on MD has none left, a point on the surrogate records this increment's F
+// at the next free position of its history (when all kmax positions are taken,
+// the last one is overwritten, so the history keeps the first kmax - 1 missed
+// increments and the latest).
+template <int NPE>
+__global__ void k_step_end(FeStepArgs a) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= a.ne) return;
+    double F[9], P[9];
+    for (int k = 0; k < 9; k++) F[k] = a.F[9 * e + k];
+    if (a.md_flag[e]) {
+        for (int k = 0; k < 9; k++) P[k] = a.P_md[9 * e + k];
+        a.n_frozen[e] = 0;
+    } else {
+        surrogate_P(a.s_mean + 6 * e, F, P);
+        const int n = a.n_frozen[e], slot = n < a.kmax ? n : a.kmax - 1;
+        for (int k = 0; k < 9; k++) a.F_hist[((size_t)slot * a.ne + e) * 9 + k] = F[k];
+        a.n_frozen[e] = n < a.kmax ? n + 1 : a.kmax;
+    }
+    for (int k = 0; k < 9; k++) {
+        a.P[9 * e + k] = P[k];
+        a.F_prev[9 * e + k] = F[k];
+    }
+    element_fint<NPE>(a.X, a.conn, a.gradN, a.V0, P, a.d, a.hg, a.fint, e);
 }
 
 }  // namespace
 
-void fe_launch_surrogate_merge(const int *md_flag, const float *s_sur, const double *F, const double *P_md, double *P,
-                               int ne, cudaStream_t s) {
-    k_merge_P<<<(ne + 127) / 128, 128, 0, s>>>(md_flag, s_sur, F, P_md, P, ne);
+void fe_launch_step_begin(int npe, const FeStepArgs &a, cudaStream_t s) {
+    if (npe == 4) k_step_begin<4><<<(a.ne + 63) / 64, 64, 0, s>>>(a);
+    else k_step_begin<8><<<(a.ne + 63) / 64, 64, 0, s>>>(a);
 }
-void fe_launch_decide(const float *spread, float on, float off, int force_md, int *md_flag, int *n_md, int ne,
-                      cudaStream_t s) {
-    k_decide<<<(ne + 127) / 128, 128, 0, s>>>(spread, on, off, force_md, md_flag, n_md, ne);
+void fe_launch_step_decide(const FeStepArgs &a, cudaStream_t s) {
+    const int n = a.ne > a.n3 ? a.ne : a.n3;
+    k_step_decide<<<(n + 127) / 128, 128, 0, s>>>(a);
+}
+void fe_launch_step_end(int npe, const FeStepArgs &a, cudaStream_t s) {
+    if (npe == 4) k_step_end<4><<<(a.ne + 63) / 64, 64, 0, s>>>(a);
+    else k_step_end<8><<<(a.ne + 63) / 64, 64, 0, s>>>(a);
 }
 void fe_launch_replay_mask(const int *md_flag, const int *n_frozen, int j, int *mask, int ne, cudaStream_t s) {
     k_replay_mask<<<(ne + 127) / 128, 128, 0, s>>>(md_flag, n_frozen, j, mask, ne);
 }
-void fe_launch_track_frozen(const int *md_flag, const double *F, double *F_hist, int *n_frozen, int ne, int kmax,
-                            cudaStream_t s) {
-    k_track_frozen<<<(ne + 127) / 128, 128, 0, s>>>(md_flag, F, F_hist, n_frozen, ne, kmax);
-}
-void fe_launch_copy_F(const double *F, double *F_prev, int ne, cudaStream_t s) {
-    k_copy_F<<<(9 * ne + 255) / 256, 256, 0, s>>>(F, F_prev, 9 * ne);
-}
-
 void fe_launch_geometry(int npe, const double *X, const int *conn, int ne, double rho0, double *gradN, double *V0,
                         double *mass, int *err, cudaStream_t s) {
     if (npe == 4) k_geometry<4><<<(ne + 127) / 128, 128, 0, s>>>(X, conn, ne, rho0, gradN, V0, mass, err);

@@ -1677,21 +1677,9 @@ __global__ void k_ensemble(const float *__restrict__ Sm, int n_members, int n, f
                            float *spread) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    float mu[NOUT], var = 0.0f, nrm = 0.0f;
-    for (int c = 0; c < NOUT; c++) {
-        float s = 0.0f;
-        for (int k = 0; k < n_members; k++) s += Sm[((size_t)k * n + i) * NOUT + c];
-        mu[c] = s / n_members;
-        float q = 0.0f;
-        for (int k = 0; k < n_members; k++) {
-            const float d = Sm[((size_t)k * n + i) * NOUT + c] - mu[c];
-            q += d * d;
-        }
-        var += n_members > 1 ? q / (n_members - 1) : 0.0f;
-        nrm += mu[c] * mu[c];
-        mean[(size_t)i * NOUT + c] = mu[c];
-    }
-    spread[i] = sqrtf(var) / fmaxf(sqrtf(nrm), s_floor);
+    float mu[NOUT];
+    spread[i] = rc_ensemble(Sm, n_members, n, i, s_floor, mu);
+    for (int c = 0; c < NOUT; c++) mean[(size_t)i * NOUT + c] = mu[c];
 }
 
 __global__ void k_h_to_input(const float *__restrict__ h, int n, __nv_bfloat16 *Z) {
@@ -1701,23 +1689,9 @@ __global__ void k_h_to_input(const float *__restrict__ h, int n, __nv_bfloat16 *
     Z[(size_t)b * K0 + NIN + k] = __float2bfloat16(h[idx]);
 }
 
-// surrogate input of one increment: u = (F - F_prev (row-major, 9), E = (F^T F - I)/2 in
-// Voigt order xx yy zz xy xz yz (6))
 __global__ void k_features(const double *__restrict__ Fp, const double *__restrict__ F, int n, float *u) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const double *f = F + 9 * i, *fp = Fp + 9 * i;
-    float *o = u + (size_t)i * NIN;
-    for (int k = 0; k < 9; k++) o[k] = (float)(f[k] - fp[k]);
-    double C[9];
-    for (int a = 0; a < 3; a++)
-        for (int b = 0; b < 3; b++) C[3 * a + b] = f[a] * f[b] + f[3 + a] * f[3 + b] + f[6 + a] * f[6 + b];
-    o[9] = (float)(0.5 * (C[0] - 1.0));
-    o[10] = (float)(0.5 * (C[4] - 1.0));
-    o[11] = (float)(0.5 * (C[8] - 1.0));
-    o[12] = (float)(0.5 * C[1]);
-    o[13] = (float)(0.5 * C[2]);
-    o[14] = (float)(0.5 * C[5]);
+    if (i < n) rc_features(Fp + 9 * i, F + 9 * i, u + (size_t)i * NIN);
 }
 
 inline int cdiv(long a, int b) { return (int)((a + b - 1) / b); }
@@ -2214,10 +2188,22 @@ int sur_predict(sur_ctx *s, const float *U, int B, int T, float *Sout) {
 }
 
 int sur_step(sur_ctx *s, const float *u, int n, float *h, float s_floor, float *s_mean, float *spread) {
-    if (!s || !u || !h || !s_mean || !spread || n <= 0 || n > s->Bmax) return RC_EINVAL;
+    if (!s || !s_mean || !spread) return RC_EINVAL;
+    const float *Sm = nullptr;
+    const int e = sur_step_members(s, u, n, h, &Sm, nullptr);
+    if (e != RC_OK) return e;
+    k_ensemble<<<cdiv(n, 128), 128, 0, s->stream>>>(Sm, s->K, n, s_floor, s_mean, spread);
+    return cudaGetLastError() == cudaSuccess ? RC_OK : RC_ECUDA;
+}
+
+}  // extern "C"
+
+int sur_step_members(sur_ctx *s, const float *u, int n, float *h, const float **Sm, int *n_members) {
+    if (!s || !u || !h || n <= 0 || n > s->Bmax) return RC_EINVAL;
+    *Sm = s->Sm;
+    if (n_members) *n_members = s->K;
     if (s->backend == 2) {
         forward_fused(s, 0, s->K, u, n, 1, s->Sm, (long)n * NOUT, NOUT, s->s_mul, h, (long)n * NH, false);
-        k_ensemble<<<cdiv(n, 128), 128, 0, s->stream>>>(s->Sm, s->K, n, s_floor, s_mean, spread);
         return cudaGetLastError() == cudaSuccess ? RC_OK : RC_ECUDA;
     }
     __nv_bfloat16 *Z = s->Z;  // n rows of [u, h, 0]
@@ -2250,9 +2236,10 @@ int sur_step(sur_ctx *s, const float *u, int n, float *h, float s_floor, float *
         if (s->backend) gemm_tc05<EPI_HEAD>(s->stream, in, WID, M.Wt[3], WID, n, N4, WID, hd, s->d_err);
         else gemm<EPI_HEAD, false>(s->stream, in, WID, M.W[3], N4, n, N4, WID, hd);
     }
-    k_ensemble<<<cdiv(n, 128), 128, 0, s->stream>>>(s->Sm, s->K, n, s_floor, s_mean, spread);
     return cudaGetLastError() == cudaSuccess ? RC_OK : RC_ECUDA;
 }
+
+extern "C" {
 
 int sur_set_backend(sur_ctx *s, int backend) {
     if (!s || backend < 0 || backend > 2) return RC_EINVAL;

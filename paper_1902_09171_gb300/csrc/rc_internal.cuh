@@ -230,6 +230,41 @@ void rc_launch_pdl(void (*kernel)(KArgs...), unsigned grid, unsigned block, size
     cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// Surrogate input of one increment: u = (F - F_prev (row-major, 9), E = (F^T F - I)/2 in
+// Voigt order xx yy zz xy xz yz (6))
+__device__ __forceinline__ void rc_features(const double *fp, const double *f, float *o) {
+    for (int k = 0; k < 9; k++) o[k] = (float)(f[k] - fp[k]);
+    double C[9];
+    for (int a = 0; a < 3; a++)
+        for (int b = 0; b < 3; b++) C[3 * a + b] = f[a] * f[b] + f[3 + a] * f[3 + b] + f[6 + a] * f[6 + b];
+    o[9] = (float)(0.5 * (C[0] - 1.0));
+    o[10] = (float)(0.5 * (C[4] - 1.0));
+    o[11] = (float)(0.5 * (C[8] - 1.0));
+    o[12] = (float)(0.5 * C[1]);
+    o[13] = (float)(0.5 * C[2]);
+    o[14] = (float)(0.5 * C[5]);
+}
+
+// Ensemble statistics of point i of n (Sm: n_members x n x 6): the members' mean
+// stress into mu, returns their relative spread
+__device__ __forceinline__ float rc_ensemble(const float *__restrict__ Sm, int n_members, int n, int i, float s_floor,
+                                             float (&mu)[6]) {
+    float var = 0.0f, nrm = 0.0f;
+    for (int c = 0; c < 6; c++) {
+        float s = 0.0f;
+        for (int k = 0; k < n_members; k++) s += Sm[((size_t)k * n + i) * 6 + c];
+        mu[c] = s / n_members;
+        float q = 0.0f;
+        for (int k = 0; k < n_members; k++) {
+            const float d = Sm[((size_t)k * n + i) * 6 + c] - mu[c];
+            q += d * d;
+        }
+        var += n_members > 1 ? q / (n_members - 1) : 0.0f;
+        nrm += mu[c] * mu[c];
+    }
+    return sqrtf(var) / fmaxf(sqrtf(nrm), s_floor);
+}
+
 // per-cell state of the FIRE minimiser (k_fire.cu)
 struct FireState {
     double *acc;      // [cell][4]: f.v, |v|^2, |f|^2, pad
@@ -287,11 +322,30 @@ void fe_launch_fint(int npe, const double *X, const int *conn, const double *gra
                     const double *d, double hg, double *fint, int ne, cudaStream_t s);
 void fe_launch_update(const int *mask, const double *mass, const double *fint, double dt, double damping,
                       double *d, double *v, int n3, cudaStream_t s);
-void fe_launch_surrogate_merge(const int *md_flag, const float *s_sur, const double *F, const double *P_md, double *P,
-                               int ne, cudaStream_t s);
-void fe_launch_decide(const float *spread, float on, float off, int force_md, int *md_flag, int *n_md, int ne,
-                      cudaStream_t s);
-void fe_launch_copy_F(const double *F, double *F_prev, int ne, cudaStream_t s);
+// one FE step with the surrogate, in three kernels around the members' forward
+// pass (see k_fe.cu)
+struct FeStepArgs {
+    int ne, n3;  // elements; 3 x nodes
+    const int *conn, *mask;
+    const double *X, *gradN, *V0, *val, *g;
+    double lambda, dlambda, hg;
+    double *d, *fint, *F, *F_prev, *P;
+    const double *P_md;
+    float *u;
+    const float *Sm;  // members' stresses, n_members x ne x 6
+    int n_members;
+    float s_floor, on, off;
+    int force_md, *md_flag, *n_frozen, kmax;
+    float *s_mean, *spread, *spread_out;
+    int *host_flag, *host_frozen;  // pinned host memory
+    double *F_hist;
+};
+void fe_launch_step_begin(int npe, const FeStepArgs &a, cudaStream_t s);
+void fe_launch_step_decide(const FeStepArgs &a, cudaStream_t s);
+void fe_launch_step_end(int npe, const FeStepArgs &a, cudaStream_t s);
 void fe_launch_replay_mask(const int *md_flag, const int *n_frozen, int j, int *mask, int ne, cudaStream_t s);
-void fe_launch_track_frozen(const int *md_flag, const double *F, double *F_hist, int *n_frozen, int ne, int kmax,
-                            cudaStream_t s);
+
+// the forward pass of sur_step (k_mlp.cu): every member's stresses at n points,
+// device, n_members x n x 6 in *Sm; h is advanced
+struct sur_ctx;
+int sur_step_members(sur_ctx *s, const float *u, int n, float *h, const float **Sm, int *n_members);

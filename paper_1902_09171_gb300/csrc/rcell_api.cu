@@ -83,12 +83,11 @@ struct fe_ctx {
     // surrogate-coupled steps (allocated on first use)
     float *d_u = nullptr, *d_smean = nullptr, *d_spread = nullptr;
     double *d_Pmd = nullptr;
-    int *d_nmd = nullptr;
     // per point: deformation gradients of the increments missed while on the
     // surrogate ([RC_REPLAY_MAX][ne][9]), their count, and a replay mask
     double *d_Fhist = nullptr;
     int *d_nfrozen = nullptr, *d_rmask = nullptr;
-    std::vector<int> h_flag, h_nfrozen;
+    int *h_flag = nullptr, *h_nfrozen = nullptr;  // pinned: this step's flags and counts, written by its kernel
     std::string err = "ok";
 };
 
@@ -1136,35 +1135,67 @@ int fe_step_surrogate(fe_ctx *fe, rcell_ctx *rc, sur_ctx *sur, double lambda, in
     }
     const int ne = fe->ne;
     cudaStream_t st = fe->stream;
-    if (!fe->d_u) {
+    if (!fe->h_flag) {
         CKF(fe, dalloc(fe->allocs, &fe->d_u, 15 * (size_t)ne));
         CKF(fe, dalloc(fe->allocs, &fe->d_smean, 6 * (size_t)ne));
         CKF(fe, dalloc(fe->allocs, &fe->d_spread, ne));
         CKF(fe, dalloc(fe->allocs, &fe->d_Pmd, 9 * (size_t)ne));
-        CKF(fe, dalloc(fe->allocs, &fe->d_nmd, 1));
         CKF(fe, dalloc(fe->allocs, &fe->d_Fhist, (size_t)RC_REPLAY_MAX * ne * 9));
         CKF(fe, dalloc(fe->allocs, &fe->d_nfrozen, ne));
         CKF(fe, dalloc(fe->allocs, &fe->d_rmask, ne));
-        fe->h_flag.assign(ne, 0);
-        fe->h_nfrozen.assign(ne, 0);
+        void *pinned = nullptr;
+        CKF(fe, cudaHostAlloc(&pinned, 2 * sizeof(int) * (size_t)ne, cudaHostAllocDefault));
+        fe->h_flag = static_cast<int *>(pinned);
+        fe->h_nfrozen = fe->h_flag + ne;
     }
     int e;
-    // 1. boundary conditions and element F
-    apply_bc(fe, lambda, st);
-    fe_launch_F(fe->npe, fe->d_conn, fe->d_gradN, fe->d_d, fe->d_F, ne, st);
+    FeStepArgs a{};
+    a.ne = ne;
+    a.n3 = 3 * fe->nn;
+    a.conn = fe->d_conn;
+    a.mask = fe->d_mask;
+    a.X = fe->d_X;
+    a.gradN = fe->d_gradN;
+    a.V0 = fe->d_V0;
+    a.val = fe->d_val;
+    a.g = fe->d_g;
+    a.lambda = lambda;
+    a.dlambda = lambda - fe->lam_last;
+    a.hg = fe->hg;
+    a.d = fe->d_d;
+    a.fint = fe->d_fint;
+    a.F = fe->d_F;
+    a.F_prev = F_prev;
+    a.P = fe->d_P;
+    a.P_md = fe->d_Pmd;
+    a.u = fe->d_u;
+    a.s_floor = s_floor;
+    a.on = spread_on;
+    a.off = spread_off;
+    a.force_md = force_md;
+    a.md_flag = md_flag;
+    a.n_frozen = fe->d_nfrozen;
+    a.kmax = RC_REPLAY_MAX;
+    a.s_mean = fe->d_smean;
+    a.spread = fe->d_spread;
+    a.spread_out = spread_out;
+    a.host_flag = fe->h_flag;
+    a.host_frozen = fe->h_nfrozen;
+    a.F_hist = fe->d_Fhist;
+    // 1. element F under this step's boundary conditions and the surrogate's input
+    fe_launch_step_begin(fe->npe, a, st);
     // 2. surrogate for every point (keeps every recurrent state current)
-    if ((e = sur_features(F_prev, fe->d_F, ne, fe->d_u, st)) != RC_OK) return e;
-    if ((e = sur_step(sur, fe->d_u, ne, h_state, s_floor, fe->d_smean, fe->d_spread)) != RC_OK) return e;
-    // 3. which points fall back to MD
-    CKF(fe, cudaMemsetAsync(fe->d_nmd, 0, sizeof(int), st));
-    fe_launch_decide(fe->d_spread, spread_on, spread_off, force_md, md_flag, fe->d_nmd, ne, st);
-    if (spread_out)
-        CKF(fe, cudaMemcpyAsync(spread_out, fe->d_spread, sizeof(float) * ne, cudaMemcpyDeviceToDevice, st));
-    int nmd = 0;
-    CKF(fe, cudaMemcpyAsync(&nmd, fe->d_nmd, sizeof(int), cudaMemcpyDeviceToHost, st));
-    CKF(fe, cudaMemcpyAsync(fe->h_flag.data(), md_flag, sizeof(int) * ne, cudaMemcpyDeviceToHost, st));
-    CKF(fe, cudaMemcpyAsync(fe->h_nfrozen.data(), fe->d_nfrozen, sizeof(int) * ne, cudaMemcpyDeviceToHost, st));
+    if ((e = sur_step_members(sur, fe->d_u, ne, h_state, &a.Sm, &a.n_members)) != RC_OK) {
+        apply_bc(fe, lambda, st);
+        return e;
+    }
+    // 3. which points fall back to MD; the displacements
+    fe_launch_step_decide(a, st);
+    fe->lam_last = lambda;
+    CKF(fe, cudaGetLastError());
     CKF(fe, cudaStreamSynchronize(st));
+    int nmd = 0;
+    for (int k = 0; k < ne; k++) nmd += fe->h_flag[k] != 0;
     // 4. a point returning to MD resumes from its frozen r-cell state (the state of
     //    its last MD increment) and first replays, increment by increment, the
     //    deformations it missed on the surrogate (R15); points replay side by side,
@@ -1193,11 +1224,9 @@ int fe_step_surrogate(fe_ctx *fe, rcell_ctx *rc, sur_ctx *sur, double lambda, in
     }
     // 6. merge: MD P where flagged, J sigma_sur F^-T elsewhere; record the missed
     //    increment of every surrogate point; then the FE update
-    fe_launch_surrogate_merge(md_flag, fe->d_smean, fe->d_F, fe->d_Pmd, fe->d_P, ne, st);
-    fe_launch_track_frozen(md_flag, fe->d_F, fe->d_Fhist, fe->d_nfrozen, ne, RC_REPLAY_MAX, st);
-    fe_launch_copy_F(fe->d_F, F_prev, ne, st);
+    fe_launch_step_end(fe->npe, a, st);
+    fe_launch_update(fe->d_mask, fe->d_mass, fe->d_fint, fe->dt, fe->damping, fe->d_d, fe->d_v, 3 * fe->nn, st);
     CKF(fe, cudaGetLastError());
-    if ((e = fe_update(fe, fe->d_P, RC_DEVICE)) != RC_OK) return e;
     if (n_md) *n_md = nmd;
     if (n_replayed) *n_replayed = replayed;
     return RC_OK;
@@ -1223,6 +1252,7 @@ void fe_destroy(fe_ctx *fe) {
     if (!fe) return;
     if (fe->stream) cudaStreamSynchronize(fe->stream);
     for (void *p : fe->allocs) cudaFree(p);
+    if (fe->h_flag) cudaFreeHost(fe->h_flag);
     if (fe->ev) cudaEventDestroy(fe->ev);
     if (fe->own_stream && fe->stream) cudaStreamDestroy(fe->stream);
     delete fe;
