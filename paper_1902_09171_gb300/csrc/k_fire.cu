@@ -9,8 +9,9 @@
 // after more than 5 such steps dt = min(1.1 dt, dt_max), alpha = 0.99 alpha;
 // p <= 0: n_pos = 0, v = 0, dt = dt / 2, alpha = 0.1; then v += dt f / m,
 // x += dt v, an atom whose move would exceed dmax (> 0) having its velocity
-// scaled to move dmax.  Kernels: k_fire_power (per-cell p, |v|^2, |f|^2, max |f|^2),
-// k_fire_control (per cell), k_fire_move (per atom).
+// scaled to move dmax.  The force kernel forms p, |v|^2, |f|^2 and max |f|^2 per cell
+// (MODE_FORCE: without virial and energy, which an iteration does not need); then
+// k_fire_control (per cell) and k_fire_move (per atom).
 #include "rc_internal.cuh"
 
 namespace {
@@ -44,43 +45,9 @@ __global__ void __launch_bounds__(RC_TILE) k_fire_zero_v(KArrays a, FireState s,
     if (li < a.cell_n[c] && go) a.v[a.cell_off[c] + li] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-__global__ void __launch_bounds__(RC_TILE) k_fire_power(KArrays a, FireState s) {
-    const int t = blockIdx.x, c = a.tile_cell[t];
-    if (s.done[c]) return;
-    const int li = (t - a.cell_tile0[c]) * RC_TILE + threadIdx.x;
-    float p = 0.f, vv = 0.f, ff = 0.f, f2max = 0.f;
-    if (li < a.cell_n[c]) {
-        const int g = a.cell_off[c] + li;
-        const float4 f = a.f[g], v = a.v[g];
-        p = f.x * v.x + f.y * v.y + f.z * v.z;
-        vv = v.x * v.x + v.y * v.y + v.z * v.z;
-        ff = f.x * f.x + f.y * f.y + f.z * f.z;
-        f2max = ff;
-    }
-    __shared__ double s_part[RC_TILE / 32][3];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) {
-        p += __shfl_xor_sync(0xffffffffu, p, d);
-        vv += __shfl_xor_sync(0xffffffffu, vv, d);
-        ff += __shfl_xor_sync(0xffffffffu, ff, d);
-        f2max = fmaxf(f2max, __shfl_xor_sync(0xffffffffu, f2max, d));
-    }
-    if (lane == 0) {
-        s_part[warp][0] = p;
-        s_part[warp][1] = vv;
-        s_part[warp][2] = ff;
-        atomicMax(&s.fmax2[c], __float_as_uint(f2max));  // non-negative floats order like their bits
-    }
-    __syncthreads();
-    if (threadIdx.x < 3) {
-        double sum = 0.0;
-        for (int w = 0; w < RC_TILE / 32; w++) sum += s_part[w][threadIdx.x];
-        atomicAdd(&s.acc[4 * c + threadIdx.x], sum);
-    }
-}
-
 __global__ void k_fire_control(FireState s, int n_cells, float f_tol2, float dt_max, int *n_left) {
+    rc_pdl_wait();
+    rc_pdl_trigger();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= n_cells || s.done[c]) return;
     const float f2max = __uint_as_float(s.fmax2[c]);
@@ -117,6 +84,8 @@ __global__ void k_fire_control(FireState s, int n_cells, float f_tol2, float dt_
 }
 
 __global__ void __launch_bounds__(RC_TILE) k_fire_move(KParams p, KArrays a, int cur, FireState s, float dmax) {
+    rc_pdl_wait();
+    rc_pdl_trigger();
     const int t = blockIdx.x, c = a.tile_cell[t];
     if (s.done[c]) return;
     const int li = (t - a.cell_tile0[c]) * RC_TILE + threadIdx.x;
@@ -225,9 +194,8 @@ void rc_launch_fire_zero_v(const KArrays &a, const FireState &s, int n_tiles, in
 
 void rc_launch_fire_iteration(const KParams &p, const KArrays &a, int cur, const FireState &s, int n_tiles, int n_cells,
                               float f_tol, float dt_max, float dmax, int *n_left, cudaStream_t st) {
-    k_fire_power<<<n_tiles, RC_TILE, 0, st>>>(a, s);
-    k_fire_control<<<(n_cells + 127) / 128, 128, 0, st>>>(s, n_cells, f_tol * f_tol, dt_max, n_left);
-    k_fire_move<<<n_tiles, RC_TILE, 0, st>>>(p, a, cur, s, dmax);
+    rc_launch_pdl(k_fire_control, (n_cells + 127) / 128, 128, 0, st, 1, s, n_cells, f_tol * f_tol, dt_max, n_left);
+    rc_launch_pdl(k_fire_move, n_tiles, RC_TILE, 0, st, 1, p, a, cur, s, dmax);
 }
 
 void rc_launch_static_prep(const double *H, const double *H0, float *mcell, double *acc, int n_cells,

@@ -350,7 +350,7 @@ __device__ __forceinline__ void block_reduce_add(float (&v)[NV], double *dst) {
 
 // What follows the sums over an atom's neighbours (force f, virial w, energy pe):
 // the embedding energy, the chain bonds, and the integration step or, in
-// MODE_EVAL, the result.  One thread per atom (own), NT threads per block;
+// MODE_EVAL and MODE_FORCE, the result.  One thread per atom (own), NT threads per block;
 // bonded[k] is the record of atom k of the cell.
 template <int POT, int NT>
 __device__ __forceinline__ void finish_atom(const KParams &p, const KArrays &a, int cur, int mode, int slot, int step_index,
@@ -412,6 +412,24 @@ __device__ __forceinline__ void finish_atom(const KParams &p, const KArrays &a, 
         float v[7] = {own ? pe : 0.f, own ? w0 : 0.f, own ? w1 : 0.f, own ? w2 : 0.f,
                       own ? w3 : 0.f, own ? w4 : 0.f, own ? w5 : 0.f};
         block_reduce_add<7, NT>(v, a.eval_acc + 8 * c);
+        return;
+    }
+
+    if (mode == MODE_FORCE) {  // the sums over the cell that decide its next FIRE move
+        float v[3] = {0.f, 0.f, 0.f};
+        if (own) {
+            const float4 vv = a.v[g];
+            a.f[g] = make_float4(fx, fy, fz, 0.0f);
+            // (explicit rounding: the minimiser's branches turn on these sums' last bits)
+            v[0] = fmaf(fz, vv.z, fmaf(fx, vv.x, __fmul_rn(fy, vv.y)));
+            v[1] = fmaf(vv.z, vv.z, fmaf(vv.x, vv.x, __fmul_rn(vv.y, vv.y)));
+            v[2] = fmaf(fz, fz, fmaf(fx, fx, __fmul_rn(fy, fy)));
+        }
+        float f2max = v[2];
+#pragma unroll
+        for (int d = 16; d >= 1; d >>= 1) f2max = fmaxf(f2max, __shfl_xor_sync(0xffffffffu, f2max, d));
+        if ((threadIdx.x & 31) == 0) atomicMax(&a.fire_fmax2[c], __float_as_uint(f2max));  // non-negative: ordered as their bits
+        block_reduce_add<3, NT>(v, a.fire_acc + 4 * c);
         return;
     }
 
@@ -487,11 +505,18 @@ constexpr int force_min_ctas(int tpa, bool sample) {
     return tpa == 0 ? (sample ? 8 : 10) : (RC_FORCE_MIN_CTAS / tpa > 0 ? RC_FORCE_MIN_CTAS / tpa : 1);
 }
 
-// SAMPLE: this launch records a stress sample (slot >= 0) or evaluates the
-// energy and virial (MODE_EVAL); without it the pair loop skips the virial and
-// energy terms, which only feed those records.
-template <int POT, int TPA, bool M6, bool STG, bool SAMPLE>
-__global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), force_min_ctas(TPA, SAMPLE)) k_force(KParams p, KArrays a, int cur, int mode, int slot,
+// WHAT the walk sums: the force alone in an MD step; force, virial and energy
+// where a stress sample is recorded (slot >= 0) or in MODE_EVAL; the force alone,
+// rounded as it is beside the virial, for the FIRE minimiser, whose branches turn
+// on the last bit of f . v (160 000 beads: 80 us per iteration with the virial and
+// a kernel of its own for the power sums, 68 us so).
+enum { SUM_STEP = 0, SUM_ALL = 1, SUM_FORCE = 2 };
+inline int what_of(int mode, int slot) {
+    return slot >= 0 || mode == MODE_EVAL ? SUM_ALL : mode == MODE_FORCE ? SUM_FORCE : SUM_STEP;
+}
+
+template <int POT, int TPA, bool M6, bool STG, int WHAT>
+__global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), force_min_ctas(TPA, WHAT == SUM_ALL)) k_force(KParams p, KArrays a, int cur, int mode, int slot,
                                                        int step_index) {
     extern __shared__ __align__(16) float4 s_cell[];
     rc_pdl_wait();
@@ -523,15 +548,17 @@ __global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), force_min_ctas(TPA, SA
         auto body = [&](const float4 &xj, const float3 &d) {
             float e;
             const float gr = pair_term<POT, M6>(p, xi, xj, d, e);
-            if (!SAMPLE) {
+            if (WHAT == SUM_STEP) {
                 fx = fmaf(gr, d.x, fx);
                 fy = fmaf(gr, d.y, fy);
                 fz = fmaf(gr, d.z, fz);
-            } else {  // w, pe: scaled once per atom after the walk
-                const float gx = gr * d.x, gy = gr * d.y, gz = gr * d.z;
-                fx = __fadd_rn(fx, gx);
-                fy = __fadd_rn(fy, gy);
-                fz = __fadd_rn(fz, gz);
+                return;
+            }
+            const float gx = gr * d.x, gy = gr * d.y, gz = gr * d.z;
+            fx = __fadd_rn(fx, gx);
+            fy = __fadd_rn(fy, gy);
+            fz = __fadd_rn(fz, gz);
+            if (WHAT == SUM_ALL) {  // w, pe: scaled once per atom after the walk
                 w0 = fmaf(gx, d.x, w0);
                 w1 = fmaf(gy, d.y, w1);
                 w2 = fmaf(gz, d.z, w2);
@@ -543,7 +570,7 @@ __global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), force_min_ctas(TPA, SA
         };
         if (STG) for_each_neighbor<TPA>(nb, nn, sub, SharedSrc{s_cell, off}, xi, s_tab, body);
         else for_each_neighbor<TPA>(nb, nn, sub, GlobalSrc{XG}, xi, s_tab, body);
-        if (SAMPLE) {
+        if (WHAT == SUM_ALL) {
             pe *= POT == RC_POT_SC ? 0.5f * p.eps : 2.0f * p.eps;
             w0 *= -0.5f;
             w1 *= -0.5f;
@@ -556,7 +583,7 @@ __global__ void __launch_bounds__(RC_TILE *lanes_of(TPA), force_min_ctas(TPA, SA
     fx = sub_sum<TPA>(fx);
     fy = sub_sum<TPA>(fy);
     fz = sub_sum<TPA>(fz);
-    if (SAMPLE) {
+    if (WHAT == SUM_ALL) {
         w0 = sub_sum<TPA>(w0);
         w1 = sub_sum<TPA>(w1);
         w2 = sub_sum<TPA>(w2);
@@ -657,10 +684,10 @@ __global__ void __launch_bounds__(COOP_THREADS, CTAS) k_density_coop(KParams p, 
     if (li < n && l == 0) a.xr[g] = make_float4(xi.x, xi.y, xi.z, rho > 0.0f ? rsqrtf(rho) : 0.0f);
 }
 
-template <int POT, bool M6, bool SAMPLE, int CTAS>
+template <int POT, bool M6, int WHAT, int CTAS>
 __global__ void __launch_bounds__(COOP_THREADS, CTAS) k_force_coop(KParams p, KArrays a, int cur, int mode, int slot, int step_index) {
     __shared__ ShiftTab s_tab;
-    __shared__ __align__(16) float s_pair[SAMPLE ? 5 : 4][COOP_COMP];  // d (3), dE/dr / r, energy: [atom][entry]
+    __shared__ __align__(16) float s_pair[WHAT == SUM_ALL ? 5 : 4][COOP_COMP];  // d (3), dE/dr / r, energy: [atom][entry]
     __shared__ float s_sum[COOP_ATOMS][11];
     rc_pdl_wait();
     rc_pdl_trigger();
@@ -681,11 +708,12 @@ __global__ void __launch_bounds__(COOP_THREADS, CTAS) k_force_coop(KParams p, KA
         const int ia = l < 3 ? l : (l < 6 ? l - 3 : (l < 8 ? 0 : 1)), ib = l < 6 ? l - 3 : (l == 6 ? 1 : 2);
         const bool f = l < 3, w = l >= 3 && l < 9;
         const int row = at * COOP_ROW;
-        const float *pa = &s_pair[l == 9 && SAMPLE ? 4 : ia][row], *pb = &s_pair[w ? ib : 0][row], *pg = &s_pair[3][row];
+        const float *pa = &s_pair[l == 9 && WHAT == SUM_ALL ? 4 : ia][row], *pb = &s_pair[w ? ib : 0][row], *pg = &s_pair[3][row];
         float acc = 0.0f;
         const auto one = [&](float gr, float da, float db) {
             const float v = gr * da;
-            if (!SAMPLE) acc = fmaf(gr, da, acc);
+            if (WHAT == SUM_STEP) acc = fmaf(gr, da, acc);
+            else if (WHAT == SUM_FORCE) acc = __fadd_rn(acc, v);
             else acc = w ? fmaf(v, db, acc) : __fadd_rn(acc, f ? v : da);
         };
         coop_walk(a.nbr + (size_t)t * p.max_nb * RC_TILE + 4 * (in0 + at), li < n ? a.nnb[g] : 0, (unsigned)g, XG, xi, s_tab,
@@ -696,16 +724,16 @@ __global__ void __launch_bounds__(COOP_THREADS, CTAS) k_force_coop(KParams p, KA
                       s_pair[1][row + l] = d.y;
                       s_pair[2][row + l] = d.z;
                       s_pair[3][row + l] = gr;
-                      if (SAMPLE) s_pair[SAMPLE ? 4 : 0][row + l] = e;
+                      if (WHAT == SUM_ALL) s_pair[WHAT == SUM_ALL ? 4 : 0][row + l] = e;
                   },
                   [&] {
-                      if (l < (SAMPLE ? 10 : 3)) {
+                      if (l < (WHAT == SUM_ALL ? 10 : 3)) {
 #pragma unroll
                           for (int k = 0; k < COOP_LANES; k += 4) {
                               const float4 gr = *reinterpret_cast<const float4 *>(pg + k),
                                            da = *reinterpret_cast<const float4 *>(pa + k);
                               float4 db = da;
-                              if (SAMPLE) db = *reinterpret_cast<const float4 *>(pb + k);
+                              if (WHAT == SUM_ALL) db = *reinterpret_cast<const float4 *>(pb + k);
                               one(gr.x, da.x, db.x);
                               one(gr.y, da.y, db.y);
                               one(gr.z, da.z, db.z);
@@ -713,14 +741,14 @@ __global__ void __launch_bounds__(COOP_THREADS, CTAS) k_force_coop(KParams p, KA
                           }
                       }
                   });
-        if (l < (SAMPLE ? 10 : 3)) s_sum[at][l] = acc;
+        if (l < (WHAT == SUM_ALL ? 10 : 3)) s_sum[at][l] = acc;
     }
     __syncthreads();
     if (threadIdx.x >= 32) return;
     const int lane = threadIdx.x, li = li0 + lane, g = off + min(li, n - 1);
     const float *r = s_sum[lane];
     float w[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (SAMPLE) {
+    if (WHAT == SUM_ALL) {
 #pragma unroll
         for (int k = 0; k < 6; k++) w[k] = -0.5f * r[3 + k];
         w[6] = (POT == RC_POT_SC ? 0.5f * p.eps : 2.0f * p.eps) * r[9];
@@ -798,25 +826,32 @@ void set_smem(K kernel, int bytes) {
     if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
-template <int POT, bool M6, bool STG, bool SAMPLE>
+template <int POT, bool M6, bool STG, int WHAT>
 void launch_force_tpa(const KParams &p, const KArrays &a, int cur, int n_tiles, int tpa, int mode, int slot,
                       int step_index, int smem, cudaStream_t s) {
     switch (tpa) {
-    case 0: rc_launch_pdl(k_force<POT, 0, M6, STG, SAMPLE>, pair_grid(p), RC_TILE * 1, smem, s, 1, p, a, cur, mode, slot, step_index); break;
-    case 1: rc_launch_pdl(k_force<POT, 1, M6, STG, SAMPLE>, pair_grid(p), RC_TILE * 1, smem, s, 1, p, a, cur, mode, slot, step_index); break;
-    case 2: rc_launch_pdl(k_force<POT, 2, M6, STG, SAMPLE>, pair_grid(p), RC_TILE * 2, smem, s, 1, p, a, cur, mode, slot, step_index); break;
-    case 4: rc_launch_pdl(k_force<POT, 4, M6, STG, SAMPLE>, pair_grid(p), RC_TILE * 4, smem, s, 1, p, a, cur, mode, slot, step_index); break;
-    default: rc_launch_pdl(k_force<POT, 8, M6, STG, SAMPLE>, pair_grid(p), RC_TILE * 8, smem, s, 1, p, a, cur, mode, slot, step_index); break;
+    case 0: rc_launch_pdl(k_force<POT, 0, M6, STG, WHAT>, pair_grid(p), RC_TILE * 1, smem, s, 1, p, a, cur, mode, slot, step_index); break;
+    case 1: rc_launch_pdl(k_force<POT, 1, M6, STG, WHAT>, pair_grid(p), RC_TILE * 1, smem, s, 1, p, a, cur, mode, slot, step_index); break;
+    case 2: rc_launch_pdl(k_force<POT, 2, M6, STG, WHAT>, pair_grid(p), RC_TILE * 2, smem, s, 1, p, a, cur, mode, slot, step_index); break;
+    case 4: rc_launch_pdl(k_force<POT, 4, M6, STG, WHAT>, pair_grid(p), RC_TILE * 4, smem, s, 1, p, a, cur, mode, slot, step_index); break;
+    default: rc_launch_pdl(k_force<POT, 8, M6, STG, WHAT>, pair_grid(p), RC_TILE * 8, smem, s, 1, p, a, cur, mode, slot, step_index); break;
     }
 }
 
 template <int POT, bool M6, bool STG>
 void launch_force_pot(const KParams &p, const KArrays &a, int cur, int n_tiles, int tpa, int mode, int slot,
                       int step_index, int smem, cudaStream_t s) {
-    if (slot >= 0 || mode == MODE_EVAL)
-        launch_force_tpa<POT, M6, STG, true>(p, a, cur, n_tiles, tpa, mode, slot, step_index, smem, s);
-    else
-        launch_force_tpa<POT, M6, STG, false>(p, a, cur, n_tiles, tpa, mode, slot, step_index, smem, s);
+    const int what = what_of(mode, slot);
+    if constexpr (!STG) {
+        if (what == SUM_FORCE) {
+            launch_force_tpa<POT, M6, STG, SUM_FORCE>(p, a, cur, n_tiles, tpa, mode, slot, step_index, smem, s);
+            return;
+        }
+    }
+    if (what == SUM_STEP)
+        launch_force_tpa<POT, M6, STG, SUM_STEP>(p, a, cur, n_tiles, tpa, mode, slot, step_index, smem, s);
+    else  // (with staging, the minimiser too)
+        launch_force_tpa<POT, M6, STG, SUM_ALL>(p, a, cur, n_tiles, tpa, mode, slot, step_index, smem, s);
 }
 
 template <bool M6, bool STG>
@@ -830,19 +865,19 @@ void launch_density_m(const KParams &p, const KArrays &a, int cur, int n_tiles, 
     }
 }
 
-template <int POT, bool M6, bool SAMPLE>
+template <int POT, bool M6, int WHAT>
 void prepare_pot_s(int bytes) {
-    set_smem(k_force<POT, 0, M6, true, SAMPLE>, bytes);
-    set_smem(k_force<POT, 1, M6, true, SAMPLE>, bytes);
-    set_smem(k_force<POT, 2, M6, true, SAMPLE>, bytes);
-    set_smem(k_force<POT, 4, M6, true, SAMPLE>, bytes);
-    set_smem(k_force<POT, 8, M6, true, SAMPLE>, bytes);
+    set_smem(k_force<POT, 0, M6, true, WHAT>, bytes);
+    set_smem(k_force<POT, 1, M6, true, WHAT>, bytes);
+    set_smem(k_force<POT, 2, M6, true, WHAT>, bytes);
+    set_smem(k_force<POT, 4, M6, true, WHAT>, bytes);
+    set_smem(k_force<POT, 8, M6, true, WHAT>, bytes);
 }
 
 template <int POT, bool M6>
 void prepare_pot(int bytes) {
-    prepare_pot_s<POT, M6, true>(bytes);
-    prepare_pot_s<POT, M6, false>(bytes);
+    prepare_pot_s<POT, M6, SUM_ALL>(bytes);
+    prepare_pot_s<POT, M6, SUM_STEP>(bytes);
 }
 
 template <bool M6>
@@ -904,10 +939,15 @@ namespace {
 template <int POT, bool M6>
 void launch_force(const KParams &p, const KArrays &a, int cur, int n_tiles, int tpa, int mode, int slot, int step_index,
                   int stage_atoms, int coop_tiles, cudaStream_t s) {
-    const bool sample = slot >= 0 || mode == MODE_EVAL;
+    const int what = what_of(mode, slot);
     if (coop_tiles > 0) {
-        const auto k = coop_two(p, coop_tiles) ? (sample ? k_force_coop<POT, M6, true, 2> : k_force_coop<POT, M6, false, 2>)
-                                               : (sample ? k_force_coop<POT, M6, true, 3> : k_force_coop<POT, M6, false, 3>);
+        const auto k = coop_two(p, coop_tiles)
+                           ? (what == SUM_ALL     ? k_force_coop<POT, M6, SUM_ALL, 2>
+                              : what == SUM_FORCE ? k_force_coop<POT, M6, SUM_FORCE, 2>
+                                                  : k_force_coop<POT, M6, SUM_STEP, 2>)
+                           : (what == SUM_ALL     ? k_force_coop<POT, M6, SUM_ALL, 3>
+                              : what == SUM_FORCE ? k_force_coop<POT, M6, SUM_FORCE, 3>
+                                                  : k_force_coop<POT, M6, SUM_STEP, 3>);
         rc_launch_pdl(k, coop_tiles * COOP_PER_TILE, COOP_THREADS, 0, s, 1, p, a, cur, mode, slot, step_index);
     } else if (stage_atoms > 0)
         launch_force_pot<POT, M6, true>(p, a, cur, n_tiles, tpa, mode, slot, step_index, stage_atoms * 16, s);

@@ -34,7 +34,8 @@
 #define RC_SAMPLE_W 14  // per-step sample record: K[6], W[6], pe, ke
 
 // per-step force-kernel modes
-enum { MODE_EVAL = 0, MODE_SETUP = 1, MODE_STEP = 2, MODE_LAST = 3 };
+// (MODE_FORCE: forces and the FIRE minimiser's power sums only)
+enum { MODE_EVAL = 0, MODE_SETUP = 1, MODE_STEP = 2, MODE_LAST = 3, MODE_FORCE = 4 };
 
 // Everything a kernel needs, passed by value.
 struct KParams {
@@ -73,6 +74,8 @@ struct KArrays {
     const unsigned long long *evals;
     double *series;      // [cell][slot][RC_SAMPLE_W]
     int series_cap;
+    double *fire_acc;    // [cell][4] and [cell]: f.v, |v|^2, |f|^2 and max |f|^2 bits (MODE_FORCE)
+    unsigned *fire_fmax2;
     double *eval_acc;    // [cell][8]: pe, W xx yy zz xy xz yz, pad
     // per atom
     float4 *x0, *x1;     // ping-pong

@@ -726,6 +726,8 @@ int rcell_minimize(rcell_ctx *c, int max_iter, double f_tol, double dt0, double 
         CKC(c, dalloc(L, &f.zero, nc));
         CKC(c, dalloc(L, &f.moving, nc));
         CKC(c, dalloc(L, &c->d_fire_left, 1));
+        c->ka.fire_acc = f.acc;
+        c->ka.fire_fmax2 = f.fmax2;
     }
     rc_launch_fire_init(c->fire, c->ka.status, c->ka.active, nc, (float)dt0, c->stream);
     rc_launch_fire_zero_v(c->ka, c->fire, c->n_tiles, 0, c->stream);
@@ -739,13 +741,14 @@ int rcell_minimize(rcell_ctx *c, int max_iter, double f_tol, double dt0, double 
         ~MaskSwap() { c->ka.active = saved; }
     } swap{c, c->ka.active};
     c->ka.active = c->fire.moving;
-    // iterations in batches between convergence checks: forces (MODE_EVAL, after the
-    // list and density kernels), then the FIRE power / control / move kernels
+    // iterations in batches between convergence checks: forces and power sums
+    // (MODE_FORCE, after the list and density kernels), then the FIRE control and
+    // move kernels
     const int batch = 32;
     auto enqueue_batch = [&](int nb) {
         cudaMemsetAsync(c->d_fire_left, 0, sizeof(int), c->stream);
         for (int k = 0; k < nb; k++) {  // the last iteration of the batch counts the cells still moving
-            enqueue_step(c, MODE_EVAL, -1, 0);
+            enqueue_step(c, MODE_FORCE, -1, 0);
             rc_launch_fire_iteration(c->kp, c->ka, c->cur, c->fire, c->n_tiles, nc, (float)f_tol, (float)dt_max,
                                      (float)dmax, k == nb - 1 ? c->d_fire_left : nullptr, c->stream);
         }
