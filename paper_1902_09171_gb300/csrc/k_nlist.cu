@@ -331,11 +331,12 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS) k_nlist(KParams p, KArray
             const float *H = a.Hf + 8 * c;
             const float4 *tab = a.shift + (size_t)c * RC_SHIFT_W;
             const int *bs = a.bin_start + a.bin_off[c];
-            // r_list, and what the bins' edges may be off: a few roundings of the box
+            // r_list, and 4e-6 of the box for what positions, bins and their edges may be
+            // off: a few roundings (6e-8 each), both to lower and to higher bins
             const float reach = sqrtf(p.rlist2) + 4e-6f * (fabsf(H[0]) + fabsf(H[1]) + fabsf(H[2]) + fabsf(H[3]) +
                                                            fabsf(H[4]) + fabsf(H[5]));
             const float r0 = 1.0f / nb0, r1 = 1.0f / nb1, r2 = 1.0f / nb2;
-            const float reach2 = reach * reach, to_bins = 1.00001f * nb2 / H[5];
+            const float reach2 = reach * reach, to_bins = nb2 / H[5];
             // entry k of atom li of the cell lives at word 4 * ((t * max_nb/4 + k/4) * TILE + at) + k%4
             const auto out = [&](int li) {
                 return reinterpret_cast<int4 *>(a.nbr) + (size_t)(t0 + li / RC_TILE) * (p.max_nb / 4) * RC_TILE + li % RC_TILE;
@@ -386,7 +387,6 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS) k_nlist(KParams p, KArray
                     int start0 = 0, len0 = 0, start1 = 0, len1 = 0, start2 = 0, len2 = 0, s0 = 0, s1 = 0;
                     if (lane < 25) {
                         const int u0 = (b01 >> 10) + o0, u1 = (b01 & 1023) + o1;
-                        
                         // extent of the row's bins (all of z that can matter) along x and y
                         const float f0 = u0 * r0, f1 = u1 * r1, f2 = (z_min - 2) * r2, e2 = (z_max + 3) * r2;
                         const float e0 = f0 + r0, e1 = f1 + r1;
