@@ -238,7 +238,7 @@ int rcell_set_staging(rcell_ctx *ctx, int staged);
  * >= dt0 > 0); dmax > 0 caps every atom's move per iteration (its velocity is
  * scaled down; <= 0: no cap).  At most max_iter iterations.  iters_out (n_cells host ints, or
  * NULL) receives each cell's number of moves before convergence (-1: not
- * converged, or skipped).  Velocities are zero afterwards.  Synchronous.
+ * converged, skipped, or failed on the way).  Velocities are zero afterwards.  Synchronous.
  * RC_EINVAL for bad arguments; cell errors as for rcell_run. */
 int rcell_minimize(rcell_ctx *ctx, int max_iter, double f_tol, double dt0, double dt_max, double dmax,
                    int *iters_out);

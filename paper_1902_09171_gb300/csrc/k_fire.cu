@@ -45,11 +45,16 @@ __global__ void __launch_bounds__(RC_TILE) k_fire_zero_v(KArrays a, FireState s,
     if (li < a.cell_n[c] && go) a.v[a.cell_off[c] + li] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-__global__ void k_fire_control(FireState s, int n_cells, float f_tol2, float dt_max, int *n_left) {
+__global__ void k_fire_control(FireState s, const int *status, int n_cells, float f_tol2, float dt_max, int *n_left) {
     rc_pdl_wait();
     rc_pdl_trigger();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= n_cells || s.done[c]) return;
+    if (status[c] != 0) {  // the pair kernels leave a failed cell out: its sums say nothing
+        s.done[c] = 1;
+        s.moving[c] = 0;
+        return;  // iters stays -1
+    }
     const float f2max = __uint_as_float(s.fmax2[c]);
     const double p = s.acc[4 * c], vv = s.acc[4 * c + 1], ff = s.acc[4 * c + 2];
     s.fmax2[c] = 0u;
@@ -194,7 +199,7 @@ void rc_launch_fire_zero_v(const KArrays &a, const FireState &s, int n_tiles, in
 
 void rc_launch_fire_iteration(const KParams &p, const KArrays &a, int cur, const FireState &s, int n_tiles, int n_cells,
                               float f_tol, float dt_max, float dmax, int *n_left, cudaStream_t st) {
-    rc_launch_pdl(k_fire_control, (n_cells + 127) / 128, 128, 0, st, 1, s, n_cells, f_tol * f_tol, dt_max, n_left);
+    rc_launch_pdl(k_fire_control, (n_cells + 127) / 128, 128, 0, st, 1, s, a.status, n_cells, f_tol * f_tol, dt_max, n_left);
     rc_launch_pdl(k_fire_move, n_tiles, RC_TILE, 0, st, 1, p, a, cur, s, dmax);
 }
 
