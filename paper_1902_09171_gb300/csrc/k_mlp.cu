@@ -1841,8 +1841,8 @@ void forward(sur_ctx *s, int k, const float *U, int B, int T, float *S, const fl
 // of member k0 + i at S + i s_ms): gradients into their grad blocks (zeroed
 // here), loss partial sums into loss_acc[k0 + i].  False when the weight-gradient
 // kernel could not be set up.
-bool backward_members(sur_ctx *s, int k0, int nk, const float *Y, int B, int T, const float *S, long s_ms,
-                      cudaEvent_t mid = nullptr) {
+[[nodiscard]] bool backward_members(sur_ctx *s, int k0, int nk, const float *Y, int B, int T, const float *S, long s_ms,
+                                    cudaEvent_t mid = nullptr) {
     const size_t RB = (size_t)B;
     cudaMemsetAsync(s->grad_all + (size_t)k0 * NPAR, 0, sizeof(float) * NPAR * nk, s->stream);
     const float gscale = 2.0f / ((float)B * T * NOUT);
@@ -2155,19 +2155,20 @@ int sur_profile_step(sur_ctx *s, const float *U, const float *Y, int B, int T, d
     for (auto &e : ev)
         if (cudaEventCreate(&e) != cudaSuccess) return RC_ECUDA;
     cudaMemsetAsync(s->loss_acc, 0, sizeof(double) * s->K, s->stream);
+    bool whole = true;  // the weight gradients were launched
     cudaEventRecord(ev[0], s->stream);
     if (s->backend == 2) {
         forward_fused(s, 0, s->K, U, B, T, s->S, s_ms, T * NOUT, nullptr, nullptr, 0, true);
         cudaEventRecord(ev[1], s->stream);
-        backward_members(s, 0, s->K, Y, B, T, s->S, s_ms, ev[2]);
+        whole = backward_members(s, 0, s->K, Y, B, T, s->S, s_ms, ev[2]);
     } else {  // per member: the phases summed over the members
         for (int k = 0; k < s->K; k++) forward(s, k, U, B, T, s->S + k * s_ms, nullptr);
         cudaEventRecord(ev[1], s->stream);
-        for (int k = 0; k < s->K; k++) backward_members(s, k, 1, Y, B, T, s->S + k * s_ms, 0);
+        for (int k = 0; k < s->K; k++) whole = backward_members(s, k, 1, Y, B, T, s->S + k * s_ms, 0) && whole;
         cudaEventRecord(ev[2], s->stream);
     }
     cudaEventRecord(ev[3], s->stream);
-    int rc = cudaEventSynchronize(ev[3]) == cudaSuccess ? RC_OK : RC_ECUDA;
+    int rc = cudaEventSynchronize(ev[3]) == cudaSuccess && whole ? RC_OK : RC_ECUDA;
     float t[3] = {0.f, 0.f, 0.f};
     for (int i = 0; i < 3 && rc == RC_OK; i++)
         if (cudaEventElapsedTime(&t[i], ev[i], ev[i + 1]) != cudaSuccess) rc = RC_ECUDA;
