@@ -155,7 +155,7 @@ __device__ __forceinline__ void eval_group(const int4 &e, const float4 &c0, cons
         d2 = rc_disp_central(xi, c2);
         d3 = rc_disp_central(xi, c3);
     } else if (__all_sync(am, (((unsigned)(e.x ^ e.y) | (unsigned)(e.x ^ e.z) | (unsigned)(e.x ^ e.w)) >> RC_IDX_BITS) == 0)) {
-        const float4 sa = T.a[s0], sb = T.b[s0];
+        const float4 sa = T.a(s0), sb = T.b(s0);
         const float4 xs = make_float4(xi.x - sb.x, xi.y - sb.y, xi.z - sb.z, sb.w);
         d0 = rc_disp_pre(c0, sa, xs);
         d1 = rc_disp_pre(c1, sa, xs);

@@ -153,7 +153,9 @@ constexpr int RC_SLOT_CENTRAL = 0;
 constexpr unsigned RC_SLOT_NULL = 27;
 constexpr int RC_SLOTS = 28, RC_SHIFT_W = 2 * RC_SLOTS;
 struct ShiftTab {
-    float4 a[RC_SLOTS], b[RC_SLOTS];
+    float4 ab[RC_SHIFT_W];  // a of every slot, then b
+    __device__ __forceinline__ const float4 &a(unsigned slot) const { return ab[slot]; }
+    __device__ __forceinline__ const float4 &b(unsigned slot) const { return ab[RC_SLOTS + slot]; }
 };
 
 __host__ __device__ __forceinline__ int rc_image_slot(int sx, int sy, int sz) {
@@ -179,7 +181,7 @@ __device__ __forceinline__ void rc_build_shift(float4 *tab, const float *H, int 
 
 // cell c's table to shared memory (call with all threads; syncs)
 __device__ __forceinline__ void rc_load_shifts(ShiftTab &T, const float4 *shift, int c) {
-    if (threadIdx.x < RC_SHIFT_W) T.a[threadIdx.x] = shift[(size_t)c * RC_SHIFT_W + threadIdx.x];
+    if (threadIdx.x < RC_SHIFT_W) T.ab[threadIdx.x] = shift[(size_t)c * RC_SHIFT_W + threadIdx.x];
     __syncthreads();
 }
 
@@ -187,13 +189,13 @@ __device__ __forceinline__ void rc_load_shifts(ShiftTab &T, const float4 *shift,
 // x_j - x_i bit for bit (rc_disp_central).  Lists hold their central entries
 // first, so the lanes of a warp walk long runs of central entries together.
 __device__ __forceinline__ float3 rc_disp(const float4 &xi, const float4 &xj, const ShiftTab &T, int slot) {
-    const float4 sa = T.a[slot], sb = T.b[slot];
+    const float4 sa = T.a(slot), sb = T.b(slot);
     return make_float3(((xj.x + sa.x) - (xi.x - sb.x)) + sa.w, ((xj.y + sa.y) - (xi.y - sb.y)) + sb.w,
                        (xj.z + sa.z) - (xi.z - sb.z));
 }
 
-// rc_disp with the slot's entries sa = T.a[slot] and xs = {x_i - T.b[slot] (3),
-// T.b[slot].w} formed once for several neighbours of the same image slot
+// rc_disp with the slot's entries sa = T.a(slot) and xs = {x_i - T.b(slot) (3),
+// T.b(slot).w} formed once for several neighbours of the same image slot
 __device__ __forceinline__ float3 rc_disp_pre(const float4 &xj, const float4 &sa, const float4 &xs) {
     return make_float3(((xj.x + sa.x) - xs.x) + sa.w, ((xj.y + sa.y) - xs.y) + xs.w, (xj.z + sa.z) - xs.z);
 }
