@@ -1,7 +1,8 @@
 // Neighbour-list build for triclinic r-cells (one list per cell, all cells of a
 // batch in one launch of each kernel).
 //
-//  k_sort  : one thread-block cluster per rebuilt r-cell.  Wraps positions into
+//  k_sort  : one thread-block cluster per rebuilt r-cell, or one CTA where many
+//            small ones rebuild.  Wraps positions into
 //            the current box through fractional coordinates, bins atoms on an
 //            n0 x n1 x n2 grid over the fractional cube (n_d = floor(2 w_d /
 //            r_list), w_d the perpendicular width: bins at least r_list / 2
@@ -59,10 +60,12 @@ __device__ __forceinline__ int compact_cells(int *s_list, int *s_warp, int n_cel
 // ---------------------------------------------------------------------------
 // k_sort.  A cluster of SORT_CL CTAs sorts one cell: the bin counters are
 // spread over the CTAs' shared memory (bin b in CTA b / per), counted with
-// atomics on distributed shared memory; the value an atomic returns is an
-// atom's arrival number in its bin, which depends on timing.  So the atoms of a
-// bin are first listed in arrival order, and each then takes its place by the
-// number of atoms of the bin that precede it in the current order: a stable,
+// atomics on distributed shared memory.  Where more cells rebuild than there are
+// clusters and they are small (spread_pays), each CTA sorts a cell of its own
+// instead, with all counters in its shared memory.  Either way the value an atomic
+// returns is an atom's arrival number in its bin, which depends on timing.  So the
+// atoms of a bin are first listed in arrival order, and each then takes its place by
+// the number of atoms of the bin that precede it in the current order: a stable,
 // deterministic order without a serial pass (bins hold a few atoms).
 // Measured per MD step: 32 cells of 5000 beads, two or three of which rebuild in
 // a step, 29.8 -> 14.7 us against one CTA per cell with a serial one-warp ranking
@@ -70,60 +73,74 @@ __device__ __forceinline__ int compact_cells(int *s_list, int *s_warp, int n_cel
 // takes 46 us, of one 256-atom cell about 15 us (six cluster barriers and their
 // dependent loads).
 // ---------------------------------------------------------------------------
-constexpr int SORT_CL = 8, SORT_THREADS = 512, SORT_SPAN = SORT_CL * SORT_THREADS;
-constexpr int SORT_BATCH = 2;  // atoms per thread whose loads are issued together
-constexpr int SORT_BINS = RC_MAX_BINS_PER_CELL / SORT_CL;
-static_assert(SORT_BINS == 2 * SORT_THREADS, "the scan takes two bins per thread");
+constexpr int SORT_CL = 8, SORT_THREADS = 512;
+constexpr int SORT_SCAN = 2 * SORT_THREADS;  // bins the block scans at a time
+static_assert(RC_MAX_BINS_PER_CELL / SORT_CL % SORT_SCAN == 0, "the scan takes whole rounds");
 
-// exclusive scan of s[0 .. 2 SORT_THREADS) in place, returns the total
-__device__ __forceinline__ int block_exclusive_scan(int *s, int *s_warp) {
+// exclusive scan of s[0 .. n) in place (n a multiple of SORT_SCAN), returns the total
+__device__ __forceinline__ int block_exclusive_scan(int *s, int n, int *s_warp) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int a = s[2 * threadIdx.x], b = s[2 * threadIdx.x + 1];
-    int v = a + b;
+    int total = 0;
+    for (int b0 = 2 * threadIdx.x; b0 < n; b0 += SORT_SCAN) {
+        const int a = s[b0], b = s[b0 + 1];
+        int v = a + b;
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, v, d);
-        if (lane >= d) v += y;
+        for (int d = 1; d < 32; d <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, v, d);
+            if (lane >= d) v += y;
+        }
+        if (lane == 31) s_warp[warp] = v;
+        __syncthreads();
+        int base = total;
+        for (int w = 0; w < SORT_THREADS / 32; w++) {
+            const int k = s_warp[w];
+            if (w < warp) base += k;
+            total += k;
+        }
+        s[b0] = base + v - a - b;
+        s[b0 + 1] = base + v - b;
+        __syncthreads();
     }
-    if (lane == 31) s_warp[warp] = v;
-    __syncthreads();
-    int base = 0, total = 0;
-    for (int w = 0; w < SORT_THREADS / 32; w++) {
-        const int k = s_warp[w];
-        if (w < warp) base += k;
-        total += k;
-    }
-    s[2 * threadIdx.x] = base + v - a - b;
-    s[2 * threadIdx.x + 1] = base + v - b;
-    __syncthreads();
     return total;
 }
 
+// Cell c, by the cluster (SPREAD; this is its CTA `rank`) or by this CTA alone;
+// BATCH atoms per thread whose loads are issued together.
+template <bool SPREAD, int BATCH>
 __device__ void sort_cell(const KParams &p, const KArrays &a, int cur, int c, int rank, int *s_cnt, int *s_warp,
                           int *s_total, cg::cluster_group &cluster) {
+    constexpr int SPAN = SPREAD ? SORT_CL * SORT_THREADS : SORT_THREADS;
+    const auto sync = [&] {
+        if constexpr (SPREAD) cluster.sync();
+        else __syncthreads();
+    };
     const int n = a.cell_n[c], off = a.cell_off[c];
     const int nb0 = a.nbins[4 * c], nb1 = a.nbins[4 * c + 1], nb2 = a.nbins[4 * c + 2];
-    const int nbt = nb0 * nb1 * nb2, per = (nbt + SORT_CL - 1) / SORT_CL;
+    const int nbt = nb0 * nb1 * nb2, per = SPREAD ? (nbt + SORT_CL - 1) / SORT_CL : nbt;  // bins of a CTA
+    const int scan = (per + SORT_SCAN - 1) / SORT_SCAN * SORT_SCAN;
     const float *H = a.Hf + 8 * c, *Hi = a.Hif + 8 * c;
     const float h00 = H[0], h01 = H[1], h02 = H[2], h11 = H[3], h12 = H[4], h22 = H[5];
     const float i00 = Hi[0], i01 = Hi[1], i02 = Hi[2], i11 = Hi[3], i12 = Hi[4], i22 = Hi[5];
     float4 *X = cur ? a.x1 : a.x0;
     const bool kg = p.pot == RC_POT_KG;
-    const int me = rank * SORT_THREADS + threadIdx.x;
+    const int me = (SPREAD ? rank * SORT_THREADS : 0) + threadIdx.x;
     int *bs = a.bin_start + a.bin_off[c];
-    const auto counter = [&](int bin) { return cluster.map_shared_rank(s_cnt, bin / per) + bin % per; };
+    const auto counter = [&](int bin) {
+        if constexpr (SPREAD) return cluster.map_shared_rank(s_cnt, bin / per) + bin % per;
+        else return s_cnt + bin;
+    };
 
-    for (int b = threadIdx.x; b < SORT_BINS; b += SORT_THREADS) s_cnt[b] = 0;
-    cluster.sync();
+    for (int b = threadIdx.x; b < scan; b += SORT_THREADS) s_cnt[b] = 0;
+    sync();
     // wrap, bin and count; a copy of every per-atom array into the staging arrays,
-    // SORT_BATCH atoms per thread at a time, all their loads issued before any store
-    for (int i0 = me; i0 < n; i0 += SORT_SPAN * SORT_BATCH) {
-        float4 xb[SORT_BATCH], vb[SORT_BATCH];
-        int tb[SORT_BATCH];
-        int4 pb[SORT_BATCH];
+    // BATCH atoms per thread at a time, all their loads issued before any store
+    for (int i0 = me; i0 < n; i0 += SPAN * BATCH) {
+        float4 xb[BATCH], vb[BATCH];
+        int tb[BATCH];
+        int4 pb[BATCH];
 #pragma unroll
-        for (int k = 0; k < SORT_BATCH; k++) {
-            const int i = i0 + k * SORT_SPAN;
+        for (int k = 0; k < BATCH; k++) {
+            const int i = i0 + k * SPAN;
             if (i < n) {
                 xb[k] = X[off + i];
                 vb[k] = a.v[off + i];
@@ -132,8 +149,8 @@ __device__ void sort_cell(const KParams &p, const KArrays &a, int cur, int c, in
             }
         }
 #pragma unroll
-        for (int k = 0; k < SORT_BATCH; k++) {
-            const int i = i0 + k * SORT_SPAN;
+        for (int k = 0; k < BATCH; k++) {
+            const int i = i0 + k * SPAN;
             if (i >= n) break;
             const int g = off + i;
             const float4 x = xb[k];
@@ -155,31 +172,33 @@ __device__ void sort_cell(const KParams &p, const KArrays &a, int cur, int c, in
             a.newpos[g] = atomicAdd(counter(bin), 1);  // arrival number, replaced by the place below
         }
     }
-    cluster.sync();
+    sync();
     // first atom of every bin: scan of the CTA's bins, plus the totals of the CTAs before
-    const int own = block_exclusive_scan(s_cnt, s_warp);
-    if (threadIdx.x == 0) *s_total = own;
-    cluster.sync();
+    const int own = block_exclusive_scan(s_cnt, scan, s_warp), bin0 = SPREAD ? rank * per : 0;
     int base = 0;
-    for (int r = 0; r < rank; r++) base += *cluster.map_shared_rank(s_total, r);
-    for (int b = threadIdx.x; b < per && rank * per + b < nbt; b += SORT_THREADS) {
+    if constexpr (SPREAD) {
+        if (threadIdx.x == 0) *s_total = own;
+        sync();
+        for (int r = 0; r < rank; r++) base += *cluster.map_shared_rank(s_total, r);
+    }
+    for (int b = threadIdx.x; b < per && bin0 + b < nbt; b += SORT_THREADS) {
         const int v = s_cnt[b] + base;
         s_cnt[b] = v;
-        bs[rank * per + b] = v;
+        bs[bin0 + b] = v;
     }
-    if (rank == 0 && threadIdx.x == 0) bs[nbt] = n;
-    cluster.sync();
+    if (bin0 == 0 && threadIdx.x == 0) bs[nbt] = n;
+    sync();
     // the atoms of every bin in arrival order
-    for (int i = me; i < n; i += SORT_SPAN) a.oldidx[off + *counter(a.binid[off + i]) + a.newpos[off + i]] = i;
-    cluster.sync();
+    for (int i = me; i < n; i += SPAN) a.oldidx[off + *counter(a.binid[off + i]) + a.newpos[off + i]] = i;
+    sync();
     // every atom to its place: the first of its bin plus the number of its
     // bin's atoms before it.  Another CTA's writes are read past the L1 cache.
-    for (int i0 = me; i0 < n; i0 += SORT_SPAN * SORT_BATCH) {
-        int bb[SORT_BATCH], tb[SORT_BATCH];
-        float4 xb[SORT_BATCH], vb[SORT_BATCH];
+    for (int i0 = me; i0 < n; i0 += SPAN * BATCH) {
+        int bb[BATCH], tb[BATCH];
+        float4 xb[BATCH], vb[BATCH];
 #pragma unroll
-        for (int k = 0; k < SORT_BATCH; k++) {
-            const int i = i0 + k * SORT_SPAN;
+        for (int k = 0; k < BATCH; k++) {
+            const int i = i0 + k * SPAN;
             if (i < n) {
                 const int g = off + i;
                 bb[k] = a.binid[g];
@@ -189,8 +208,8 @@ __device__ void sort_cell(const KParams &p, const KArrays &a, int cur, int c, in
             }
         }
 #pragma unroll
-        for (int k = 0; k < SORT_BATCH; k++) {
-            const int i = i0 + k * SORT_SPAN;
+        for (int k = 0; k < BATCH; k++) {
+            const int i = i0 + k * SPAN;
             if (i >= n) break;
             const int lo = __ldcg(bs + bb[k]), hi = __ldcg(bs + bb[k] + 1);
             int q = lo;
@@ -206,21 +225,21 @@ __device__ void sort_cell(const KParams &p, const KArrays &a, int cur, int c, in
         }
     }
     if (kg) {  // bonded partners renumbered
-        cluster.sync();
-        for (int i0 = me; i0 < n; i0 += SORT_SPAN * SORT_BATCH) {
-            int4 pb[SORT_BATCH];
-            int qb[SORT_BATCH];
+        sync();
+        for (int i0 = me; i0 < n; i0 += SPAN * BATCH) {
+            int4 pb[BATCH];
+            int qb[BATCH];
 #pragma unroll
-            for (int k = 0; k < SORT_BATCH; k++) {
-                const int i = i0 + k * SORT_SPAN;
+            for (int k = 0; k < BATCH; k++) {
+                const int i = i0 + k * SPAN;
                 if (i < n) {
                     pb[k] = a.partner_tmp[off + i];
                     qb[k] = a.newpos[off + i];
                 }
             }
 #pragma unroll
-            for (int k = 0; k < SORT_BATCH; k++) {
-                const int i = i0 + k * SORT_SPAN;
+            for (int k = 0; k < BATCH; k++) {
+                const int i = i0 + k * SPAN;
                 if (i < n) {
                     const int4 pr = pb[k];
                     const int *np = a.newpos + off;
@@ -231,24 +250,75 @@ __device__ void sort_cell(const KParams &p, const KArrays &a, int cur, int c, in
             }
         }
     }
-    cluster.sync();  // no CTA's counters change while another one reads them
+    sync();  // no CTA's counters change while another one reads them
 }
 
+// Whether n_go cells are sorted sooner by the n_cl clusters, in turn, than by one
+// CTA each (the CTAs in turn, and no sooner than the largest cell): the same answer
+// in every CTA.  Times of one cell in us: by a cluster 9 + 0.8 per thousand atoms,
+// by a CTA 6 + 5.  A sort of all cells, all by clusters / as chosen here: 64 cells of
+// 256 atoms 28 / 12 us, 1024 of 256 457 / 37, 48 of 2048 29 / 19, 48 of 4000 31 / 28
+// (clusters), 256 of 4000 149 / 40, 1024 of 500 beads 598 / 48; a step of 1024 cells of
+// 256 atoms, 44 of which rebuild in it, 111 / 97.
+__device__ __forceinline__ bool spread_pays(const KArrays &a, const int *s_list, int n_go, int n_cl, int *s_warp, int *s_max) {
+    int sum = 0, top = 0;
+    for (int k = threadIdx.x; k < n_go; k += SORT_THREADS) {
+        const int n = a.cell_n[s_list[k]];
+        sum += n;
+        top = max(top, n);
+    }
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) {
+        sum += __shfl_xor_sync(0xffffffffu, sum, d);
+        top = max(top, __shfl_xor_sync(0xffffffffu, top, d));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        s_warp[threadIdx.x >> 5] = sum;
+        s_max[threadIdx.x >> 5] = top;
+    }
+    __syncthreads();
+    sum = top = 0;
+    for (int w = 0; w < SORT_THREADS / 32; w++) {
+        sum += s_warp[w];
+        top = max(top, s_max[w]);
+    }
+    __syncthreads();
+    const int n_ctas = n_cl * SORT_CL;
+    const float mean = (float)sum / n_go;
+    const float spread = ((n_go + n_cl - 1) / n_cl) * (9.0f + 0.8e-3f * mean);
+    const float alone = fmaxf(((n_go + n_ctas - 1) / n_ctas) * (6.0f + 5e-3f * mean), 6.0f + 5e-3f * top);
+    return spread <= alone;
+}
+
+// MANY: a batch of more cells than there are clusters, none of more atoms than a
+// cluster has threads.  It has both ways to sort a cell, at one atom per thread
+// and without a spill (at two it spills more than the other one, 64 cells of 5000 to
+// 20 000 beads run 1 % longer); the other one has clusters only.
+template <bool MANY>
 __global__ void __launch_bounds__(SORT_THREADS, 2) k_sort(KParams p, KArrays a, int cur, int n_cells) {
-    __shared__ int s_cnt[SORT_BINS], s_list[LIST_CAP], s_warp[SORT_THREADS / 32], s_total;
+    __shared__ int s_cnt[MANY ? RC_MAX_BINS_PER_CELL : RC_MAX_BINS_PER_CELL / SORT_CL];
+    __shared__ int s_list[LIST_CAP], s_warp[SORT_THREADS / 32], s_max[SORT_THREADS / 32], s_total;
     rc_pdl_wait();
     rc_pdl_trigger();
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = blockIdx.x % SORT_CL, id = blockIdx.x / SORT_CL, n_cl = gridDim.x / SORT_CL;
+    int next = blockIdx.x;  // this CTA's next cell to sort alone
     // the cells to rebuild: the same list in every CTA (k_nlist, after this
-    // kernel, clears their flags), dealt to the clusters in turn
+    // kernel, clears their flags), dealt to the clusters or CTAs in turn
     for (int from = 0; from < n_cells; from += LIST_CAP) {
         const int n_go = compact_cells(s_list, s_warp, n_cells, from, [&](int c) {
             const bool go = a.need_rebuild[c] && a.status[c] == 0 && a.active[c];
             if (blockIdx.x == 0) a.built[c] = go;
             return go;
         });
-        for (int k = id; k < n_go; k += n_cl) sort_cell(p, a, cur, s_list[k], rank, s_cnt, s_warp, &s_total, cluster);
+        if (!MANY || n_go <= n_cl || spread_pays(a, s_list, n_go, n_cl, s_warp, s_max)) {
+            for (int k = id; k < n_go; k += n_cl)
+                sort_cell<true, MANY ? 1 : 2>(p, a, cur, s_list[k], rank, s_cnt, s_warp, &s_total, cluster);
+        } else {
+            for (; next < n_go; next += gridDim.x)
+                sort_cell<false, 1>(p, a, cur, s_list[next], 0, s_cnt, s_warp, &s_total, cluster);
+            next -= n_go;
+        }
         __syncthreads();
     }
 }
@@ -545,7 +615,8 @@ __global__ void __launch_bounds__(NL_THREADS, NL_CTAS) k_nlist(KParams p, KArray
 void rc_launch_sort(const KParams &p, const KArrays &a, int cur, int n_cells, cudaStream_t s) {
     // as many clusters as two CTAs per SM allow, at most one per cell
     const int n_cl = min(n_cells, max(1, 2 * p.n_sm / SORT_CL));
-    rc_launch_pdl(k_sort, n_cl * SORT_CL, SORT_THREADS, 0, s, SORT_CL, p, a, cur, n_cells);
+    const bool many = n_cells > n_cl && p.max_cell <= SORT_CL * SORT_THREADS;
+    rc_launch_pdl(many ? k_sort<true> : k_sort<false>, n_cl * SORT_CL, SORT_THREADS, 0, s, SORT_CL, p, a, cur, n_cells);
 }
 
 void rc_launch_nlist(const KParams &p, const KArrays &a, int cur, int n_cells, cudaStream_t s) {

@@ -52,6 +52,7 @@ struct KParams {
     int max_nb;
     float max_step;       // > 0: displacement limit per step
     int n_tiles;          // tiles of RC_TILE atoms in the batch
+    int max_cell;         // atoms of its largest cell
     int n_sm;             // SMs of the device (tile order of the pair kernels)
     int wait_polls;       // polls of a bounded device-side wait before it gives up
     int masked;           // cells are switched off: the pair kernels take their tiles from act_tiles

@@ -322,6 +322,7 @@ int rcell_create(const rcell_params *params, int n_cells, const rcell_init *cell
     c->max_nb_alloc = max_nb;
     kp.wait_polls = RC_WAIT_POLLS_DEFAULT;
     kp.n_tiles = c->n_tiles;
+    kp.max_cell = c->max_cell;
     kp.n_sm = 1;
     CKC(c, cudaDeviceGetAttribute(&kp.n_sm, cudaDevAttrMultiProcessorCount, c->device));
     if (kp.n_sm < 1) kp.n_sm = 1;
