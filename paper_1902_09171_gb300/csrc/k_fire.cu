@@ -49,8 +49,10 @@ __global__ void k_fire_control(FireState s, const int *status, int n_cells, floa
     rc_pdl_wait();
     rc_pdl_trigger();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n_cells || s.done[c]) return;
-    if (status[c] != 0) {  // the pair kernels leave a failed cell out: its sums say nothing
+    if (c >= n_cells) return;
+    const int failed = status[c];  // (loaded beside the flag, not after it)
+    if (s.done[c]) return;
+    if (failed) {  // the pair kernels leave a failed cell out: its sums say nothing
         s.done[c] = 1;
         s.moving[c] = 0;
         return;  // iters stays -1
