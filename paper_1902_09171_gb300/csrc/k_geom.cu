@@ -111,20 +111,26 @@ __device__ bool deform_cell(int c, const double *__restrict__ Fin, double *H, do
     return true;
 }
 
-// one warp per cell: lane 0 the deformation, then lane k entry k of the new box's shift table
-constexpr int DEFORM_WARPS = 4;
-__global__ void __launch_bounds__(32 * DEFORM_WARPS)
+// per_block cells per block, as many as one block per SM takes, at most a warp's:
+// lane k of the first warp the deformation of cell k, then the block's threads the
+// entries of the new boxes' shift tables.  The deformation is a chain of FP64
+// arithmetic, as long for a warp as for a lane: with a warp for every cell, 4096
+// cells took 126 us, 27 to a warp take 32 (1024 cells 42 / 28, one 26 either way).
+constexpr int DEFORM_THREADS = 128, DEFORM_CELLS = 32;
+__global__ void __launch_bounds__(DEFORM_THREADS)
     k_deform(const double *__restrict__ Fin, double *H, double *Rprev, double *Qo, double *Ro, double *Fst, double *dR,
              const double *__restrict__ H0, float *Hf, float *Hif, float4 *shift, int *status, int *need_rebuild,
-             int *nbins, const int *bin_cap, const int *active, double rlist, int n_cells) {
-    const int c = blockIdx.x * DEFORM_WARPS + threadIdx.x / 32, lane = threadIdx.x & 31;
-    if (c >= n_cells) return;
-    int done = 0;
-    if (lane == 0)
-        done = deform_cell(c, Fin, H, Rprev, Qo, Ro, Fst, dR, H0, Hf, Hif, status, need_rebuild, nbins, bin_cap, active,
-                           rlist);
-    __syncwarp();
-    if (__shfl_sync(0xffffffffu, done, 0) && lane < RC_SLOTS) rc_build_shift(shift + (size_t)c * RC_SHIFT_W, Hf + 8 * c, lane);
+             int *nbins, const int *bin_cap, const int *active, double rlist, int n_cells, int per_block) {
+    __shared__ bool s_done[DEFORM_CELLS];
+    const int c0 = blockIdx.x * per_block, n = min(per_block, n_cells - c0), t = threadIdx.x;
+    if (t < n)
+        s_done[t] = deform_cell(c0 + t, Fin, H, Rprev, Qo, Ro, Fst, dR, H0, Hf, Hif, status, need_rebuild, nbins, bin_cap,
+                                active, rlist);
+    __syncthreads();
+    for (int k = t; k < n * RC_SLOTS; k += DEFORM_THREADS) {
+        const int c = c0 + k / RC_SLOTS;
+        if (s_done[k / RC_SLOTS]) rc_build_shift(shift + (size_t)c * RC_SHIFT_W, Hf + 8 * c, k % RC_SLOTS);
+    }
 }
 
 __global__ void k_shift(const float *Hf, float4 *shift, int c) {
@@ -303,10 +309,12 @@ __global__ void k_advance(unsigned long long *evals, const int *active, int n_ce
 
 void rc_launch_deform_impl(const double *F, double *H, double *Rprev, double *Q, double *R, double *Fst, double *dR,
                            const double *H0, float *Hf, float *Hif, float4 *shift, int *status, int *need_rebuild,
-                           int *nbins, const int *bin_cap, const int *active, double rlist, int n_cells,
+                           int *nbins, const int *bin_cap, const int *active, double rlist, int n_cells, int n_sm,
                            cudaStream_t s) {
-    k_deform<<<(n_cells + DEFORM_WARPS - 1) / DEFORM_WARPS, 32 * DEFORM_WARPS, 0, s>>>(
-        F, H, Rprev, Q, R, Fst, dR, H0, Hf, Hif, shift, status, need_rebuild, nbins, bin_cap, active, rlist, n_cells);
+    const int per_block = min(DEFORM_CELLS, (n_cells + n_sm - 1) / n_sm);
+    k_deform<<<(n_cells + per_block - 1) / per_block, DEFORM_THREADS, 0, s>>>(
+        F, H, Rprev, Q, R, Fst, dR, H0, Hf, Hif, shift, status, need_rebuild, nbins, bin_cap, active, rlist, n_cells,
+        per_block);
 }
 
 void rc_launch_shift(const float *Hf, float4 *shift, int c, cudaStream_t s) { k_shift<<<1, 32, 0, s>>>(Hf, shift, c); }

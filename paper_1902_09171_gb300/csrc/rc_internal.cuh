@@ -297,7 +297,8 @@ int rc_stage_max_atoms();
 void rc_prepare_staged(int max_cell_atoms);
 void rc_launch_deform_impl(const double *F, double *H, double *Rprev, double *Q, double *R, double *Fst, double *dR,
                            const double *H0, float *Hf, float *Hif, float4 *shift, int *status, int *need_rebuild,
-                           int *nbins, const int *bin_cap, const int *active, double rlist, int n_cells, cudaStream_t s);
+                           int *nbins, const int *bin_cap, const int *active, double rlist, int n_cells, int n_sm,
+                           cudaStream_t s);
 // the shift table of cell c from its box
 void rc_launch_shift(const float *Hf, float4 *shift, int c, cudaStream_t s);
 void rc_launch_remap(const KArrays &a, const double *dR, int cur, int n_tiles, cudaStream_t s);

@@ -448,7 +448,7 @@ int rcell_create(const rcell_params *params, int n_cells, const rcell_init *cell
     CKC(c, cudaMemcpy(c->d_Fin, hI.data(), sizeof(double) * 9 * n_cells, cudaMemcpyHostToDevice));
     // initial box: the deformation kernel with F = I sets H = H0, the FP32 box copies and the bins
     rc_launch_deform_impl(c->d_Fin, c->d_H, c->d_Rprev, c->d_Q, c->d_R, c->d_F, c->d_dR, c->d_H0, c->d_Hf, c->d_Hif, c->d_shift,
-                          A.status, A.need_rebuild, c->d_nbins, c->d_bin_cap, A.active, c->rlist, n_cells, c->stream);
+                          A.status, A.need_rebuild, c->d_nbins, c->d_bin_cap, A.active, c->rlist, n_cells, kp.n_sm, c->stream);
     CKC(c, cudaGetLastError());
     int st = first_status(c);
     if (st != RC_OK) {
@@ -472,7 +472,8 @@ int rcell_set_deformation(rcell_ctx *c, const double *F, int where) {
         return fail(c, RC_EINVAL, "where");
     }
     rc_launch_deform_impl(dF, c->d_H, c->d_Rprev, c->d_Q, c->d_R, c->d_F, c->d_dR, c->d_H0, c->d_Hf, c->d_Hif, c->d_shift,
-                          c->ka.status, c->ka.need_rebuild, c->d_nbins, c->d_bin_cap, c->ka.active, c->rlist, c->n_cells, c->stream);
+                          c->ka.status, c->ka.need_rebuild, c->d_nbins, c->d_bin_cap, c->ka.active, c->rlist,
+                          c->n_cells, c->kp.n_sm, c->stream);
     rc_launch_remap(c->ka, c->d_dR, c->cur, c->n_tiles, c->stream);
     CKC(c, cudaGetLastError());
     return RC_OK;
@@ -912,7 +913,8 @@ int rcell_profile_kernels(rcell_ctx *c, int n_steps, double *ms_out) {
     // coupling kernels once: re-apply the current F (Delta R = I), then the stress reduction
     CKC(c, cudaEventRecord(ev[0], c->stream));
     rc_launch_deform_impl(c->d_F, c->d_H, c->d_Rprev, c->d_Q, c->d_R, c->d_F, c->d_dR, c->d_H0, c->d_Hf, c->d_Hif, c->d_shift,
-                          c->ka.status, c->ka.need_rebuild, c->d_nbins, c->d_bin_cap, c->ka.active, c->rlist, c->n_cells, c->stream);
+                          c->ka.status, c->ka.need_rebuild, c->d_nbins, c->d_bin_cap, c->ka.active, c->rlist,
+                          c->n_cells, c->kp.n_sm, c->stream);
     CKC(c, cudaEventRecord(ev[1], c->stream));
     rc_launch_remap(c->ka, c->d_dR, c->cur, c->n_tiles, c->stream);
     CKC(c, cudaEventRecord(ev[2], c->stream));
