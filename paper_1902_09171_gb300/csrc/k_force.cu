@@ -262,7 +262,8 @@ __device__ __forceinline__ float pair_term(const KParams &p, const float4 &xi, c
             arm = sr2 * sr2 * sr2;                     // (a/r)^6
             arn = arm * sr2 * (p.sigma * rsqrtf(r2));  // (a/r)^9
         } else {
-            arm = powf(sr2, 0.5f * p.sc_m);
+            // (zero beyond the cutoff by themselves: a negative exponent gives infinity there)
+            arm = r2 < p.rc2 ? powf(sr2, 0.5f * p.sc_m) : 0.0f;
             arn = r2 < p.rc2 ? powf(sr2, 0.5f * p.sc_n) : 0.0f;
         }
         e = arn;
