@@ -878,25 +878,27 @@ int rcell_restore(rcell_ctx *c, int cell, const void *buf, size_t bytes) {
     memcpy(&nn, p + 8, 8);
     if (magic != 0x52434B5054303031ull || nn != n) return fail(c, RC_EINVAL, "checkpoint does not match this cell");
     p += 16;
-    CKC(c, cudaStreamSynchronize(c->stream));
+    // all on the context's stream, so that the shift table is made from the box copied
+    // before it (a stream of the caller's may not wait for the default one)
     float4 *X = c->cur ? c->ka.x1 : c->ka.x0;
-    CKC(c, cudaMemcpy(X + off, p, sizeof(float4) * n, cudaMemcpyHostToDevice)); p += sizeof(float4) * n;
-    CKC(c, cudaMemcpy(c->ka.v + off, p, sizeof(float4) * n, cudaMemcpyHostToDevice)); p += sizeof(float4) * n;
-    CKC(c, cudaMemcpy(c->ka.tag + off, p, sizeof(int) * n, cudaMemcpyHostToDevice)); p += sizeof(int) * n;
-    CKC(c, cudaMemcpy(c->ka.partner + off, p, sizeof(int4) * n, cudaMemcpyHostToDevice)); p += sizeof(int4) * n;
+    CKC(c, cudaMemcpyAsync(X + off, p, sizeof(float4) * n, cudaMemcpyHostToDevice, c->stream)); p += sizeof(float4) * n;
+    CKC(c, cudaMemcpyAsync(c->ka.v + off, p, sizeof(float4) * n, cudaMemcpyHostToDevice, c->stream)); p += sizeof(float4) * n;
+    CKC(c, cudaMemcpyAsync(c->ka.tag + off, p, sizeof(int) * n, cudaMemcpyHostToDevice, c->stream)); p += sizeof(int) * n;
+    CKC(c, cudaMemcpyAsync(c->ka.partner + off, p, sizeof(int4) * n, cudaMemcpyHostToDevice, c->stream)); p += sizeof(int4) * n;
     for (double *dst : {c->d_H, c->d_Rprev, c->d_Q, c->d_R, c->d_F}) {
-        CKC(c, cudaMemcpy(dst + 9 * cell, p, sizeof(double) * 9, cudaMemcpyHostToDevice));
+        CKC(c, cudaMemcpyAsync(dst + 9 * cell, p, sizeof(double) * 9, cudaMemcpyHostToDevice, c->stream));
         p += sizeof(double) * 9;
     }
-    CKC(c, cudaMemcpy(c->d_Hf + 8 * cell, p, sizeof(float) * 8, cudaMemcpyHostToDevice)); p += sizeof(float) * 8;
-    CKC(c, cudaMemcpy(c->d_Hif + 8 * cell, p, sizeof(float) * 8, cudaMemcpyHostToDevice)); p += sizeof(float) * 8;
-    CKC(c, cudaMemcpy(c->d_nbins + 4 * cell, p, sizeof(int) * 4, cudaMemcpyHostToDevice)); p += sizeof(int) * 4;
-    CKC(c, cudaMemcpy(c->d_evals + cell, p, sizeof(unsigned long long), cudaMemcpyHostToDevice));
+    CKC(c, cudaMemcpyAsync(c->d_Hf + 8 * cell, p, sizeof(float) * 8, cudaMemcpyHostToDevice, c->stream)); p += sizeof(float) * 8;
+    CKC(c, cudaMemcpyAsync(c->d_Hif + 8 * cell, p, sizeof(float) * 8, cudaMemcpyHostToDevice, c->stream)); p += sizeof(float) * 8;
+    CKC(c, cudaMemcpyAsync(c->d_nbins + 4 * cell, p, sizeof(int) * 4, cudaMemcpyHostToDevice, c->stream)); p += sizeof(int) * 4;
+    CKC(c, cudaMemcpyAsync(c->d_evals + cell, p, sizeof(unsigned long long), cudaMemcpyHostToDevice, c->stream));
     rc_launch_shift(c->d_Hf, c->d_shift, cell, c->stream);
     CKC(c, cudaGetLastError());
     const int one = 1, zero = 0;
-    CKC(c, cudaMemcpy(c->ka.need_rebuild + cell, &one, sizeof(int), cudaMemcpyHostToDevice));
-    CKC(c, cudaMemcpy(c->ka.status + cell, &zero, sizeof(int), cudaMemcpyHostToDevice));
+    CKC(c, cudaMemcpyAsync(c->ka.need_rebuild + cell, &one, sizeof(int), cudaMemcpyHostToDevice, c->stream));
+    CKC(c, cudaMemcpyAsync(c->ka.status + cell, &zero, sizeof(int), cudaMemcpyHostToDevice, c->stream));
+    CKC(c, cudaStreamSynchronize(c->stream));  // `buf` is the caller's again
     return RC_OK;
 }
 
