@@ -196,8 +196,10 @@ int rcell_clear_status(rcell_ctx *ctx);
  *                      resident warps per SM (pays on large batches).
  *                      With 0 and 1, batches (or active cells, where the host
  *                      gave the mask) of few atoms are walked by sixteen lanes
- *                      per atom that add in the same order: the same results
- *                      bit for bit
+ *                      per atom that add in the same order: the same forces
+ *                      and trajectories bit for bit (sums over a cell --
+ *                      energy, virial, sampled stress -- are FP64 atomics,
+ *                      whose order differs)
  *   use_graphs       : 0/1, capture rcell_run into CUDA graphs
  * All settings give the same results up to summation order. */
 int rcell_set_tuning(rcell_ctx *ctx, int threads_per_atom, int use_graphs);

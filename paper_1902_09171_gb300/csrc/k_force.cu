@@ -909,7 +909,9 @@ void rc_prepare_staged(int max_cell_atoms) {
 // idle.  us per MD step, one lane / cooperative: LJ copper 18 / 14 (28 tiles),
 // 37 / 21 (70), 43 / 33 (140), 49 / 47 (280), 52 / 58 (420); Sutton-Chen 67 / 32
 // (64), 99 / 68 (224), 110 / 95 (320), 140 / 177 (640); Kremer-Grest 32 / 18 (80),
-// 46 / 40 (240), 47 / 46 (320), 52 / 64 (480).
+// 46 / 40 (240), 47 / 46 (320), 52 / 64 (480).  One line for the three potentials,
+// where LJ and Kremer-Grest cross; Sutton-Chen crosses between 320 and 640 tiles, so
+// just above the line it runs a tenth longer than it could.
 int rc_coop_max_tiles(int n_sm) { return 2 * n_sm; }
 
 namespace {
