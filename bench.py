@@ -162,10 +162,10 @@ class ClockSampler:
 
 # DRAM bytes (read + write) of one k_force<SC> launch on this workload (128 000
 # atoms, skin 1.5 A), from an ncu capture (the variant without a stress sample; the
-# other one reads the same list; profiles/k_force_k_density_sc_copper_bar.md): 121.93
-# MB read + 3.99 MB written.  Mostly the Verlet list, re-read from DRAM every
+# other one reads the same list; profiles/k_force_k_density_sc_copper_bar.md): 122.36
+# MB read + 4.79 MB written.  Mostly the Verlet list, re-read from DRAM every
 # launch.
-K_FORCE_DRAM_BYTES = 125.92e6
+K_FORCE_DRAM_BYTES = 127.16e6
 
 
 def fp32_unit_peak_tflops():
@@ -199,12 +199,12 @@ KG_BAR_SKINS, KG_BAR_TPAS = (0.3, 0.4, 0.5, 0.6, 0.8), (0, 1, 2)
 NECK_TUNE_CELLS = 128  # a quarter of the bar: 20 000 tiles, enough waves to behave like the whole
 
 # DRAM bytes (read + write) per bead of one k_force<KG> launch (the lean walk,
-# non-sampling variant), by Verlet skin, from ncu captures of 16 cells of 20 000
-# beads (mean of two launches; profiles/k_nlist_k_force_kg_16x20000.md): skin 0.4:
-# 138.67 + 4.39 MB, skin 0.5: 151.48 + 3.60 MB.  A launch's traffic grows in
+# non-sampling variant), by Verlet skin, from ncu captures of 16 necking-bar cells
+# (320 000 beads; mean of two launches; profiles/k_force_kg_necking_bar_16x20000.md):
+# skin 0.4: 146.77 + 4.55 MB, skin 0.5: 160.23 + 4.81 MB.  A launch's traffic grows in
 # proportion to its beads (lists, positions and velocities are per bead); the
 # list length depends on the skin.
-K_FORCE_KG_DRAM_BYTES_PER_ATOM = {0.4: 143.06e6 / 320000, 0.5: 155.08e6 / 320000}
+K_FORCE_KG_DRAM_BYTES_PER_ATOM = {0.4: 151.33e6 / 320000, 0.5: 165.04e6 / 320000}
 
 
 def kg_algorithmic_flops_per_atom_step(rho, bonds_per_atom):
